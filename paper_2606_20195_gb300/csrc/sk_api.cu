@@ -1050,6 +1050,7 @@ sk_status sk_solve_precond(sk_plan p, const float* A, int64_t lda, int64_t n, co
   const SolveLayout Lo = solve_layout(p->d, n, p->rule, 0);  // the offset of R does not depend on the tree
   L.R = reinterpret_cast<const double*>((char*)p->solve_buf + Lo.R);
   L.ldr = n + 1;
+  L.X = reinterpret_cast<double*>((char*)p->solve_buf + Lo.part) + n;
   L.u = base;
   L.v = base + m;
   L.w = L.v + nv;

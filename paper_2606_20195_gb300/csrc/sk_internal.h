@@ -162,6 +162,7 @@ struct LsqrLaunch {
   double *v, *w, *y, *p, *z, *x0;  // n each
   double* x;        // out: n
   double* sc;       // kLsqrScalars
+  double* X;        // n x (n+1): R^{-1} and its transpose (the QR's partial-sum scratch, free after it)
 };
 // Start (x0 from the FP32 sketch-and-solve solution; r0 = b - A x0; first step), one iteration, and
 // x = x0 + R^{-1} y.
