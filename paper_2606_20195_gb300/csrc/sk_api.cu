@@ -825,11 +825,12 @@ sk_status sk_materialize_S(sk_plan p, int64_t i0, int64_t cnt, int32_t* rows, in
 }
 
 // Solve scratch layout (bytes, each region 256-byte aligned):
-//   Y_A (d*n elements), Y_b (d elements), part (n + n*(n+1) doubles), R (n*(n+1) doubles),
-//   bcast (n doubles), bar (grid-barrier counters), status (1 word), kappa (1 double).
+//   Y_A (d*n elements), Y_b (d elements), part (n + n*(n+1) doubles: the QR's reduction buffers, then
+//   LSQR's R^-1), R (n*(n+1) doubles), tail (n doubles more for the reduction buffers, which may use R's
+//   region too), bar (grid-barrier counters), status (1 word), kappa (1 double).
 namespace {
 struct SolveLayout {
-  size_t ya, yb, part, R, bcast, bar, status, kappa, stack[2], total;
+  size_t ya, yb, part, R, tail, bar, status, kappa, stack[2], total;
 };
 size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 // stack_groups: groups of the first tree level (0: the sketch is factored by one launch).
@@ -841,7 +842,7 @@ SolveLayout solve_layout(int64_t d, int64_t n, int32_t rule, int64_t stack_group
   L.yb = off; off = al256(off + es * (size_t)d);
   L.part = off; off = al256(off + 8 * (size_t)(n + n * (n + 1)));
   L.R = off; off = al256(off + 8 * (size_t)(n * (n + 1)));
-  L.bcast = off; off = al256(off + 8 * (size_t)n);
+  L.tail = off; off = al256(off + 8 * (size_t)n);
   L.bar = off; off = al256(off + solve_bar_bytes());
   L.status = off; off = al256(off + 4);
   L.kappa = off; off = al256(off + 8);
@@ -881,8 +882,10 @@ sk_status solve_backend(sk_plan_s* p, const void* SA, int64_t lda_sa, const void
   L.rule = p->rule;
   L.src_fp64 = 0;
   L.n = n;
+  // The QR's reduction buffers may spread over the R region behind `part` (R is written at the end).
   L.part = (double*)(base + Lo.part);
-  L.bcast = (double*)(base + Lo.bcast);
+  L.part_doubles = (int64_t)(Lo.bar - Lo.part) / 8;
+  L.part_own = (int64_t)(Lo.R - Lo.part) / 8;
   L.bar = (unsigned*)(base + Lo.bar);
   L.status = (unsigned*)(base + Lo.status);
   L.kappa = (double*)(base + Lo.kappa);

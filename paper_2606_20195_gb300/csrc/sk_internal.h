@@ -119,9 +119,10 @@ struct SolveLaunch {
   int32_t src_fp64 = 0;  // 1: SA and Sb are FP64 (a stack of [R | c] factors of a tree level)
   int32_t solve_x = 1;   // 1: back substitution into x and kappa; 0: write [R | c] only (zero below the diagonal)
   int64_t d, n;
-  double* part;     // scratch: partial sums, (ncta) * (n + 2) doubles
+  double* part;     // scratch of the panel reductions, part_doubles doubles
+  int64_t part_doubles = 0;  // its size, the plan's own R region included where that follows it
+  int64_t part_own = 0;      // its size before that region
   double* R;        // scratch: n x (n+1) doubles (R and Q^T Sb)
-  double* bcast;    // scratch: n doubles
   unsigned* bar;    // scratch: solve_bar_bytes() of barrier counters, zeroed by the launcher
   unsigned* status; // sticky status word
   double* kappa;    // out: max|R_ii| / min|R_ii|
