@@ -38,6 +38,7 @@ using namespace sk;
 
 namespace sk {
 sk_status noalloc_read_status(unsigned* out);  // sk_noalloc.cu
+size_t noalloc_P_bytes();                      // chunk-total bytes its static array holds
 }
 
 struct sk_plan_s {
@@ -133,6 +134,7 @@ sk_status plan_grow(sk_plan_s* p, T** ptr, size_t* cur, size_t bytes, const char
 // Tile-kernel configuration for a plan and a column count.
 struct TileCfg {
   int32_t NC = 0, kb = 0, threads = 0, grid = 0, slices = 1, depth = 1, mb = 1;
+  int32_t long_slices = 1;  // slices without fill_slices: for callers short of chunk-total scratch
   int64_t R = 0;
   bool serial = false;
   bool lr = false;
@@ -183,6 +185,23 @@ int32_t choose_slices(const sk_plan_s* p, int64_t rows, int64_t R, int64_t ncg, 
   return (int32_t)best;
 }
 
+// More slices per chunk where `slices` of them give fewer work items than the GPU holds CTAs: as many as
+// fit in one round of CTAs, of at least 64 rows each. Below that size an item costs its CTA's start and its
+// flush of d x NC floats, and its rows hardly count; a 153rd item would cost a second round. Where one
+// slice needs no chunk totals (`finishes` false), only from three slices on, which pay for adding them up
+// (two were 2 us slower at 5000 x 256, d = 4096, k = 4). Measured, all slices at least 4096 rows / filled up
+// (and, but for the register kernel, one launch that finishes the chunk totals itself): 16384 x 16,
+// d = 256, k = 4 (4 items / 152): 42 / 14.5 us; 50001 x 33, d = 1056, k = 4 (16 / 144): 175 / 55;
+// 65536 x 64, d = 1024, k = 4 (32 / 144, register kernel): 47 / 28; 8192 x 64, d = 8192, k = 4: 43 / 28.
+int32_t fill_slices(const sk_plan_s* p, int64_t rows, int64_t R, int64_t ncg, int64_t nbg, int32_t cps,
+                    const DevInfo& di, int32_t slices, bool finishes) {
+  const int64_t first = ((p->row_offset % R) + R) % R;
+  const int64_t per = (first + rows + R - 1) / R * ncg * nbg;
+  const int64_t fit = std::min((int64_t)di.sms * std::max(cps, 1) / per, std::max<int64_t>(1, std::min(R, rows) / 64));
+  if (fit <= slices || (!finishes && slices == 1 && fit < 3)) return slices;
+  return (int32_t)fit;
+}
+
 // Owner-kernel configuration (atomic mode, SK_KERNEL_OWNER): blocks per item kb = 2 when two blocks
 // of 32-column lines fit in shared memory, else 1; false if the kernel does not apply.
 bool choose_own(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& di, bool tma_ok, TileCfg* cfg) {
@@ -203,7 +222,7 @@ bool choose_own(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& di, 
   cfg->threads = own_threads();
   cfg->grid = 0;
   cfg->R = R;
-  cfg->slices = choose_slices(p, rows, R, ncg, nbg, cps, di);
+  cfg->slices = cfg->long_slices = choose_slices(p, rows, R, ncg, nbg, cps, di);
   cfg->depth = 1;
   cfg->mb = 1;
   cfg->serial = false;
@@ -250,7 +269,8 @@ bool choose_reg(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& di, 
   cfg->kb = p->k;
   cfg->threads = reg_threads();
   cfg->R = R;
-  cfg->slices = choose_slices(p, rows, R, ncg, ntg, 1, di);
+  cfg->long_slices = choose_slices(p, rows, R, ncg, ntg, 1, di);
+  cfg->slices = fill_slices(p, rows, R, ncg, ntg, 1, di, cfg->long_slices, true);
   cfg->reg = true;
   cfg->reg_nsub = nsub;
   cfg->reg_cap = cap;
@@ -296,7 +316,8 @@ sk_status choose_tile(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo
       cfg->threads = threads;
       cfg->grid = 0;
       cfg->R = R;
-      cfg->slices = choose_slices(p, rows, R, 1, nbg, cps, di);
+      cfg->long_slices = choose_slices(p, rows, R, 1, nbg, cps, di);
+      cfg->slices = fill_slices(p, rows, R, 1, nbg, cps, di, cfg->long_slices, false);
       cfg->depth = 1;
       cfg->mb = 1;
       cfg->serial = false;
@@ -368,12 +389,13 @@ sk_status choose_tile(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo
   int32_t depth = 1;
   while (depth < kMaxRingDepth && tile_smem_bytes(p->B, kb, NC, threads, p->k, depth + 1, mb) <= optin) ++depth;
   int64_t R = p->R > 0 ? p->R : default_chunk_rows(p->m);
-  int32_t slices = 1;
+  int32_t slices = 1, long_slices = 1;
   if (!serial) {
     const int64_t ncg = (n + NC - 1) / NC;
     const int64_t nbg = (p->k + kb - 1) / kb;
     const int32_t cps = tile_ctas_per_sm(p->rule, threads, tile_smem_bytes(p->B, kb, NC, threads, p->k, depth, mb));
-    slices = choose_slices(p, rows, R, ncg, nbg, cps, di);
+    long_slices = choose_slices(p, rows, R, ncg, nbg, cps, di);
+    slices = fill_slices(p, rows, R, ncg, nbg, cps, di, long_slices, false);
   }
   cfg->NC = NC;
   cfg->kb = kb;
@@ -381,6 +403,7 @@ sk_status choose_tile(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo
   cfg->grid = serial ? 1 : 0;
   cfg->R = R;
   cfg->slices = slices;
+  cfg->long_slices = long_slices;
   cfg->depth = depth;
   cfg->mb = mb;
   cfg->lr = lr;
@@ -527,6 +550,20 @@ sk_status enqueue_sketch(sk_plan_s* p, const void* A, int64_t lda, int64_t n, in
   }
   L.status = p->dstatus;
   L.P = nullptr;
+  if (cfg.slices > 1 && cfg.long_slices == 1 && !cfg.glob && !cfg.reg) {
+    // One launch, as with one slice per chunk, which needs no chunk totals: taken where these would have
+    // to be allocated and the scratch limit or a stream capture forbids it.
+    L.fuse_finish = zero_y ? 1 : 0;
+    const size_t needP = sizeof(float) * (size_t)launch_P_floats(L);
+    if (p->tileP_bytes < needP) {
+      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+      const bool free = cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+      if (!free || (p->scratch_limit > 0 &&
+                    plan_scratch_bytes(p) - p->tileP_bytes + needP > (size_t)p->scratch_limit))
+        L.slices = cfg.slices = 1;
+    }
+    if (cfg.slices == 1) L.fuse_finish = 0;
+  }
   if (cfg.slices > 1 || cfg.glob || cfg.reg) {
     const size_t needP = sizeof(float) * (size_t)launch_P_floats(L);
     if (p->tileP_bytes < needP) {
@@ -537,7 +574,7 @@ sk_status enqueue_sketch(sk_plan_s* p, const void* A, int64_t lda, int64_t n, in
     }
     L.P = p->tileP;
   }
-  if (zero_y) {
+  if (zero_y && !L.fuse_finish) {
     cudaError_t ez = cudaMemsetAsync(Y, 0, elem_size(p->rule) * (size_t)(p->d * n), st);
     if (ez != cudaSuccess) return cuda_fail(ez, "zeroing Y");
   }
@@ -1286,6 +1323,11 @@ sk_status noalloc_tile_launch(const sk_plan_s* p, const float* A, int64_t lda, i
   L->threads = cfg.threads;
   L->grid = cfg.grid;
   L->slices = cfg.slices;
+  // One slice per chunk needs no chunk totals: taken where they would not fit in the static array.
+  if (cfg.slices > 1 && cfg.long_slices == 1 && !cfg.glob && !cfg.reg) {
+    L->fuse_finish = 1;
+    if (sizeof(float) * (size_t)launch_P_floats(*L) > noalloc_P_bytes()) L->fuse_finish = 0, L->slices = 1;
+  }
   L->depth = cfg.depth;
   L->mb = cfg.mb;
   L->lr = cfg.lr ? 1 : 0;

@@ -35,6 +35,7 @@ struct TileLaunch {
   int32_t glob = 0;   // 1: global-accumulator kernel (chunk totals in P, any d); needs P
   int32_t reg = 0;    // 1: register kernel (FP32 A through TMA, 32 columns x 1024 output rows per item); needs P
   int32_t reg_nsub = 0, reg_cap = 0;  // register kernel: TMA copies per staged box, list entries per output row
+  int32_t fuse_finish = 0;  // 1: tile kernel with slices > 1 as one cooperative launch that also writes all of Y
   int32_t no_finish = 0;  // 1: leave the chunk totals in P (no chunk-finish launch); P is then the caller's
 };
 
@@ -63,7 +64,7 @@ void tile_geometry(const TileLaunch& L, int64_t* chunks, int32_t* ncg, int32_t* 
 // Passes of the global-accumulator kernel: column slabs of *ns columns and batches of *cb chunks,
 // chosen so that the chunk totals of one pass (cb x d x ns FP32) stay resident in L2.
 void global_passes(const TileLaunch& L, int64_t* ns, int64_t* cb);
-// FP32 elements of chunk-total scratch P a launch needs (0: none).
+// FP32 elements of chunk-total scratch P a launch needs (0: none), with the barrier words of fuse_finish.
 int64_t launch_P_floats(const TileLaunch& L);
 // The global-accumulator kernel and its chunk finish, in passes (sk_global.cu); needs L.P.
 cudaError_t launch_global(const TileLaunch& L, cudaStream_t st, int32_t* launches);

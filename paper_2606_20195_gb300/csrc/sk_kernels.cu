@@ -113,6 +113,8 @@ cudaError_t launch_tile(const TileLaunch& L, cudaStream_t st, int32_t* launches)
   P.items = chunks * P.slices * P.ncg * P.nbg;
   P.acc_floats = (int32_t)tile_acc_floats((uint32_t)B, L.kb, P.D.S, L.NC);
   P.P = L.P;
+  P.chunks = chunks;
+  P.bar = nullptr;
   P.status = L.status;
   P.D.col_off = L.col_off;
   P.D.a_type = L.a_type;
@@ -150,6 +152,14 @@ cudaError_t launch_tile(const TileLaunch& L, cudaStream_t st, int32_t* launches)
   int64_t grid = L.grid > 0 ? L.grid : (int64_t)sms * per_sm;
   grid = std::min<int64_t>(grid, P.items);
   if (grid < 1) grid = 1;
+  if (L.fuse_finish && P.slices > 1) {
+    P.bar = reinterpret_cast<unsigned*>(L.P + chunks * L.d * L.n);
+    void* args[2] = {&P, &tmap};
+    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kern), dim3((unsigned)grid), dim3(L.threads), args,
+                                    smem, st);
+    if (launches) *launches += 1;
+    return e;
+  }
   kern<<<(unsigned)grid, L.threads, smem, st>>>(P, tmap);
   if (launches) *launches += 1;
   e = cudaGetLastError();
@@ -160,27 +170,35 @@ cudaError_t launch_tile(const TileLaunch& L, cudaStream_t st, int32_t* launches)
 
 // ------------------------------------------------------------------ chunk finish
 // One thread per output quad (row, 4 columns): the chunks of the launch in ascending order (finish_quad).
-template <int RULE>
+template <int RULE, int AHEAD>
 __global__ void __launch_bounds__(256) chunk_finish_kernel(const TileDesc D, float* P, int64_t t_first, int64_t chunks) {
   const int64_t nq = (D.n + 3) >> 2;
   const int64_t d = (int64_t)D.B * D.k;
   const int64_t dn = d * D.n;
   for (int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; f < d * nq; f += (int64_t)gridDim.x * blockDim.x) {
     const int64_t r = f / nq;
-    finish_quad<RULE>(D, (uint32_t)r, 4 * (f - r * nq), P, t_first, chunks, dn);
+    finish_quad<RULE, AHEAD>(D, (uint32_t)r, 4 * (f - r * nq), P, t_first, chunks, dn);
   }
+}
+
+// Few quads leave the GPU waiting for each chunk's load: four at a time there (200000 x 100, d = 1600: 96 ->
+// 94 us in all). With many, the added registers cost more than the latency (8192 x 1024, d = 2048: 25 -> 27 us).
+template <int RULE>
+static void chunk_finish_launch(const TileDesc& D, float* P, int64_t t_first, int64_t chunks, cudaStream_t st) {
+  const int64_t quads = (int64_t)D.B * D.k * ((D.n + 3) >> 2);
+  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((quads + 255) / 256, 1 << 16));
+  if (quads <= 65536) chunk_finish_kernel<RULE, 4><<<grid, 256, 0, st>>>(D, P, t_first, chunks);
+  else chunk_finish_kernel<RULE, 1><<<grid, 256, 0, st>>>(D, P, t_first, chunks);
 }
 
 cudaError_t launch_chunk_finish(const TileDesc& D, int32_t rule, float* P, int64_t t_first, int64_t chunks,
                                 cudaStream_t st, int32_t* launches) {
-  const int64_t quads = (int64_t)D.B * D.k * ((D.n + 3) >> 2);
-  const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((quads + 255) / 256, 1 << 16));
   switch (rule) {
-    case kRN: chunk_finish_kernel<kRN><<<grid, 256, 0, st>>>(D, P, t_first, chunks); break;
-    case kSR: chunk_finish_kernel<kSR><<<grid, 256, 0, st>>>(D, P, t_first, chunks); break;
-    case kDither: chunk_finish_kernel<kDither><<<grid, 256, 0, st>>>(D, P, t_first, chunks); break;
-    case kBF16: chunk_finish_kernel<kBF16><<<grid, 256, 0, st>>>(D, P, t_first, chunks); break;
-    default: chunk_finish_kernel<kFP32><<<grid, 256, 0, st>>>(D, P, t_first, chunks); break;
+    case kRN: chunk_finish_launch<kRN>(D, P, t_first, chunks, st); break;
+    case kSR: chunk_finish_launch<kSR>(D, P, t_first, chunks, st); break;
+    case kDither: chunk_finish_launch<kDither>(D, P, t_first, chunks, st); break;
+    case kBF16: chunk_finish_launch<kBF16>(D, P, t_first, chunks, st); break;
+    default: chunk_finish_launch<kFP32>(D, P, t_first, chunks, st); break;
   }
   if (launches) *launches += 1;
   return cudaGetLastError();

@@ -12,6 +12,7 @@ sk_status noalloc_tile_launch(const sk_plan_s* p, const float* A, int64_t lda, i
 size_t noalloc_elem_size(const sk_plan_s* p);
 void noalloc_record(sk_plan_s* p, int64_t launches, int64_t R, int32_t kernel);
 sk_status noalloc_read_status(unsigned* out);
+size_t noalloc_P_bytes();
 }  // namespace sk
 
 using namespace sk;
@@ -47,7 +48,7 @@ extern "C" SK_API sk_status sk_apply_noalloc(sk_plan p, const float* A, int64_t 
   s = scratch_address(&base);
   if (s != SK_OK) return s;
   const size_t need_P = sizeof(float) * (size_t)launch_P_floats(L);
-  if (kStatusBytes + need_P > kScratchBytes)
+  if (need_P > noalloc_P_bytes())
     return set_error(SK_ERR_UNSUPPORTED,
                      "sk_apply_noalloc: this size needs %zu bytes of scratch, above the %zu-byte static array; "
                      "use sk_apply",
@@ -68,6 +69,8 @@ extern "C" SK_API sk_status sk_apply_noalloc(sk_plan p, const float* A, int64_t 
                  L.glob ? SK_KERNEL_GLOBAL : L.reg ? SK_KERNEL_REGISTER : L.own ? SK_KERNEL_OWNER : SK_KERNEL_TILE);
   return SK_OK;
 }
+
+size_t sk::noalloc_P_bytes() { return kScratchBytes - kStatusBytes; }
 
 // The status word of the last no-allocation call on the current device (the first word of the
 // static array; the caller synchronizes first). A symbol copy: allocates nothing.

@@ -62,6 +62,8 @@ struct TileGrid {
   unsigned* status;            // sticky status word (kStatus*), may be null
   int32_t use_tma;             // 1: A arrives through the tensor map
   int32_t depth;               // TMA ring slots per warp
+  int64_t chunks;              // chunks of the launch
+  unsigned* bar;               // cooperative launch: two zero counters of the grid barrier; null: no finish here
 };
 
 // Per-warp TMA staging ring: `depth` slots of RB x NC floats (128-byte aligned) and their mbarriers.
@@ -647,7 +649,9 @@ __device__ __forceinline__ void emit_quad(const TileDesc& D, uint32_t r, int64_t
 // in ascending chunk order, read the chunk total from P (chunk-major, d x n each), clear it, scale,
 // quantize and add it into Y with the rule's arithmetic (binary32 add or binary16 add, round to
 // nearest), then write Y back once. Chunk totals that are zero in all four columns add nothing.
-template <int RULE>
+// FRESH: Y holds nothing yet (it counts as +0 and every quad is written). AHEAD: chunk totals whose loads
+// are in flight together (one at a time, each costs an L2 round trip).
+template <int RULE, int AHEAD, bool FRESH = false>
 __device__ __forceinline__ void finish_quad(const TileDesc& D, uint32_t r, int64_t col0, float* P, int64_t t_first,
                                             int64_t chunks, int64_t dn) {
   const int64_t n = D.n;
@@ -657,45 +661,56 @@ __device__ __forceinline__ void finish_quad(const TileDesc& D, uint32_t r, int64
   const int64_t offy = (int64_t)r * (D.ldy > 0 ? D.ldy : n) + col0;  // in Y
   float yf[4] = {0.f, 0.f, 0.f, 0.f};
   uint16_t yh[4] = {0, 0, 0, 0};
-  bool loaded = false, touched = false;
-  for (int64_t tl = 0; tl < chunks; ++tl) {
-    float* p = P + tl * dn + off;
-    float4 v;
-    if (vec) {
-      v = __ldcg(reinterpret_cast<const float4*>(p));
-    } else {
-      v.x = __ldcg(p);
-      v.y = ne > 1 ? __ldcg(p + 1) : 0.f;
-      v.z = ne > 2 ? __ldcg(p + 2) : 0.f;
-      v.w = ne > 3 ? __ldcg(p + 3) : 0.f;
-    }
-    if (v.x == 0.f && v.y == 0.f && v.z == 0.f && v.w == 0.f) continue;
-    if (vec) {
-      __stcg(reinterpret_cast<float4*>(p), make_float4(0.f, 0.f, 0.f, 0.f));
-    } else {
-      for (int e = 0; e < ne; ++e) __stcg(p + e, 0.f);
-    }
-    if (!loaded) {
-      loaded = true;
-      if (RULE == kFP32) {
-        const float* y = reinterpret_cast<const float*>(D.Y) + offy;
-        for (int e = 0; e < ne; ++e) yf[e] = y[e];
-      } else {
-        const uint16_t* y = reinterpret_cast<const uint16_t*>(D.Y) + offy;
-        for (int e = 0; e < ne; ++e) yh[e] = y[e];
-      }
-    }
-    float x[4];
-    uint16_t q[4];
-    scale_quad<RULE>(D, r, col0, v, t_first + tl, x, q);
+  bool loaded = FRESH, touched = FRESH;
+  for (int64_t tb = 0; tb < chunks; tb += AHEAD) {
+    float4 va[AHEAD];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      if (e < ne) {
-        if (RULE == kFP32) yf[e] = __fadd_rn(yf[e], x[e]);
-        else yh[e] = add16<RULE>(yh[e], q[e]);
+    for (int i = 0; i < AHEAD; ++i) {
+      const float* p = P + (tb + i) * dn + off;
+      va[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (tb + i < chunks) {
+        if (vec) {
+          va[i] = __ldcg(reinterpret_cast<const float4*>(p));
+        } else {
+          va[i].x = __ldcg(p);
+          if (ne > 1) va[i].y = __ldcg(p + 1);
+          if (ne > 2) va[i].z = __ldcg(p + 2);
+          if (ne > 3) va[i].w = __ldcg(p + 3);
+        }
       }
     }
-    touched = true;
+#pragma unroll
+    for (int i = 0; i < AHEAD; ++i) {
+      const float4 v = va[i];
+      if (v.x == 0.f && v.y == 0.f && v.z == 0.f && v.w == 0.f) continue;
+      float* p = P + (tb + i) * dn + off;
+      if (vec) {
+        __stcg(reinterpret_cast<float4*>(p), make_float4(0.f, 0.f, 0.f, 0.f));
+      } else {
+        for (int e = 0; e < ne; ++e) __stcg(p + e, 0.f);
+      }
+      if (!loaded) {
+        loaded = true;
+        if (RULE == kFP32) {
+          const float* y = reinterpret_cast<const float*>(D.Y) + offy;
+          for (int e = 0; e < ne; ++e) yf[e] = y[e];
+        } else {
+          const uint16_t* y = reinterpret_cast<const uint16_t*>(D.Y) + offy;
+          for (int e = 0; e < ne; ++e) yh[e] = y[e];
+        }
+      }
+      float x[4];
+      uint16_t q[4];
+      scale_quad<RULE>(D, r, col0, v, t_first + tb + i, x, q);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (e < ne) {
+          if (RULE == kFP32) yf[e] = __fadd_rn(yf[e], x[e]);
+          else yh[e] = add16<RULE>(yh[e], q[e]);
+        }
+      }
+      touched = true;
+    }
   }
   if (!touched) return;
   if (RULE == kFP32) {

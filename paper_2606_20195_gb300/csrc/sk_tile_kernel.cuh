@@ -8,6 +8,35 @@ namespace sk {
 
 // ------------------------------------------------------------------ tile kernel
 
+// Wait until every CTA of a co-resident (cooperative) grid has arrived; bar[0] counts arrivals, bar[1]
+// departures, and the last CTA to depart clears both for the next launch. Writes before the call are
+// visible to every CTA after it. Gives up after about two seconds (then false, and the status word says so).
+__device__ __forceinline__ bool tile_grid_barrier(unsigned* bar, unsigned* status) {
+  __shared__ int ok;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ok = 0;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    const long long t0 = clock64();
+    while (clock64() - t0 < (4ll << 30)) {
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+      if (v >= gridDim.x) {
+        ok = 1;
+        break;
+      }
+    }
+    if (!ok && status) atomicOr(status, kStatusTimeout);
+    if (ok && atomicAdd(bar + 1, 1u) == gridDim.x - 1) {
+      bar[0] = 0u;
+      bar[1] = 0u;
+    }
+  }
+  __syncthreads();
+  return ok != 0;
+}
+
 // One CTA per SM (or per work item), work items in a grid-stride loop: scatter, then flush into Y or
 // into the chunk totals. TA is the element type of A; the FP32 instantiations live in sk_kernels.cu,
 // the 16-bit ones in sk_kernels_a16.cu (compiled in parallel).
@@ -51,10 +80,22 @@ __global__ void __launch_bounds__(1024) tile_kernel(const TileGrid P, const __gr
     if (P.slices == 1) {
       tile_flush<RULE>(D, t, g, j0, kbe, acc);
     } else {
-      // slice partials into the chunk totals; chunk_finish_kernel adds them into Y after this launch
+      // slice partials into the chunk totals; the end of this kernel (P.bar) or chunk_finish_kernel after
+      // it adds them into Y
       tile_flush_partial(D, g, j0, kbe, acc, P.P + tl * dn);
     }
     __syncthreads();
+  }
+  // One-launch form for sketches too small for a second one: once every CTA's partials are in, the grid
+  // finishes the chunk totals itself and writes all of Y. At 16384 x 16, d = 256, k = 4, FP32 the separate
+  // finish and the zeroing of Y took 7 of 20 us.
+  if (P.bar) {
+    if (!tile_grid_barrier(P.bar, P.status)) return;
+    const int64_t nq = (D.n + 3) >> 2, quads = (int64_t)D.B * D.k * nq;
+    for (int64_t f = (int64_t)threadIdx.x * gridDim.x + blockIdx.x; f < quads; f += (int64_t)gridDim.x * blockDim.x) {
+      const int64_t r = f / nq;
+      finish_quad<RULE, 4, true>(D, (uint32_t)r, 4 * (f - r * nq), P.P, P.t_first, P.chunks, dn);
+    }
   }
 }
 
