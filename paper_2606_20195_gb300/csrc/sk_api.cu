@@ -141,7 +141,7 @@ struct TileCfg {
   bool own = false;
   bool vec = false;
   bool glob = false;
-  bool reg = false;
+  bool reg = false, reg_tile = false;
   int32_t reg_nsub = 0, reg_cap = 0;
 };
 
@@ -243,43 +243,48 @@ void choose_global(const sk_plan_s* p, TileCfg* cfg) {
   cfg->glob = true;
 }
 
-// Register-kernel configuration (atomic mode, FP32 A staged through TMA): the staged box and list
+// Register-kernel configuration (atomic mode, A staged through TMA): the staged box and list
 // capacity for the plan's block height, the default chunk length and the slice count. AUTO takes it
 // for k >= 2, n >= 32 and blocks of at most 512 rows (not n >= 256 with k = 2, which goes to the
 // global kernel), where it is faster than the tile kernel
 // (measured at 2^22 x 64: d = 4096, k = 8: 1060 vs 818 GB/s; d = 1024, k = 8: 1520 vs 798; at
-// d = 4096 with k = 4 or 2 (B = 1024, 2048) the tile kernel stays ahead: 1416 vs 1357, 1735 vs 1448).
-bool choose_reg(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& di, bool tma_ok, bool a_fp32,
+// d = 4096 with k = 4 or 2 (B = 1024, 2048) the tile kernel stays ahead: 1416 vs 1357, 1735 vs 1448;
+// bfloat16 A: d = 4096, k = 8: 765 vs 1332 us; d = 1024, k = 4: 287 vs 735; 2^21 x 40, d = 320, k = 4:
+// 162 vs 356; 20000 x 128, d = 2048, k = 4: 26 vs 34; 2^18 x 1024, d = 2048, k = 4: 546 vs 917).
+// `reg_tile`: the tile kernel is the one to fall back to where chunk totals cannot be had (it may need none).
+bool choose_reg(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& di, bool tma_ok, int32_t a_type,
                 TileCfg* cfg) {
-  if (p->mode != SK_MODE_ATOMIC || !tma_ok || !a_fp32 || rows >= ((int64_t)1 << 31)) return false;
+  if (p->mode != SK_MODE_ATOMIC || !tma_ok || rows >= ((int64_t)1 << 31)) return false;
   if (p->kernel == SK_KERNEL_AUTO) {
     if (p->tile_cols != 0 || p->threads != 0 || p->k < 2 || n < 32 || p->B > 512) return false;
     if (n >= 256 && p->k <= 2) return false;  // the global kernel's case (wide rows, few nonzeros)
-  } else if (p->kernel != SK_KERNEL_REGISTER) {
+  } else if (p->kernel != SK_KERNEL_REGISTER || a_type != SK_A_FP32) {
     return false;
   }
   const size_t optin = (size_t)std::min(di.optin, 232448) - 1024;
   int32_t nsub = 0, cap = 0;
-  if (!reg_choose_box(p->d, p->B, optin, p->list_cap, &nsub, &cap)) return false;
+  if (!reg_choose_box(p->d, p->B, a_type, optin, p->list_cap, &nsub, &cap)) return false;
   const int64_t R = p->R > 0 ? p->R : default_chunk_rows(p->m);
-  const int64_t ncg = (n + 31) / 32;
-  const int64_t ntg = (p->d + reg_targets() - 1) / reg_targets();
+  const int64_t ncg = (n + reg_cols(a_type) - 1) / reg_cols(a_type);
+  const int64_t ntg = (p->d + reg_targets(a_type) - 1) / reg_targets(a_type);
   *cfg = TileCfg();
   cfg->NC = 32;
   cfg->kb = p->k;
-  cfg->threads = reg_threads();
+  cfg->threads = reg_threads(a_type);
   cfg->R = R;
   cfg->long_slices = choose_slices(p, rows, R, ncg, ntg, 1, di);
   cfg->slices = fill_slices(p, rows, R, ncg, ntg, 1, di, cfg->long_slices, true);
   cfg->reg = true;
+  cfg->reg_tile = p->kernel == SK_KERNEL_AUTO && a_type != SK_A_FP32;
   cfg->reg_nsub = nsub;
   cfg->reg_cap = cap;
   return true;
 }
 
 sk_status choose_tile(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& di, TileCfg* cfg,
-                      bool tma_ok = false, bool a_fp32 = true) {
-  if (choose_reg(p, n, rows, di, tma_ok, a_fp32, cfg)) return SK_OK;
+                      bool tma_ok = false, int32_t a_type = SK_A_FP32, bool scratch = true) {
+  if (choose_reg(p, n, rows, di, tma_ok, a_type, cfg) && (scratch || !cfg->reg_tile)) return SK_OK;
+  *cfg = TileCfg();
   if (p->kernel == SK_KERNEL_REGISTER)
     return set_error(SK_ERR_UNSUPPORTED,
                      "register kernel: needs atomic mode, FP32 A, A 16-byte aligned with lda %% 4 == 0 and fewer "
@@ -428,6 +433,17 @@ sk_status validate_apply(const sk_plan_s* p, const void* A, int64_t lda, int64_t
   return SK_OK;
 }
 
+// Whether the chunk totals of a sketch with chunk length R are in place or may be allocated: within the
+// scratch limit, and not while the stream is being captured.
+bool totals_available(const sk_plan_s* p, int64_t n, int64_t row_begin, int64_t row_end, int64_t R, cudaStream_t st) {
+  const int64_t chunks = (row_end - 1) / R - row_begin / R + 1;
+  const size_t need = sizeof(float) * (size_t)(chunks * p->d * n + kBarrierFloats);
+  if (p->tileP_bytes >= need) return true;
+  if (p->scratch_limit > 0 && plan_scratch_bytes(p) - p->tileP_bytes + need > (size_t)p->scratch_limit) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+}
+
 // Enqueue Y = S * A for rows [row_begin, row_begin + rows) (A row 0 = row_begin) with chunk rows R.
 // Y must already be zero, or zero_y set: then Y is zeroed on the stream once the plan's scratch is in
 // place (a call refused for lack of scratch leaves Y untouched). a_type: element type of A
@@ -507,8 +523,13 @@ sk_status enqueue_sketch(sk_plan_s* p, const void* A, int64_t lda, int64_t n, in
     return SK_OK;
   }
   TileCfg cfg;
-  s = choose_tile(p, n, rows, di, &cfg, tma_layout_ok(A, lda, a_type == SK_A_FP32 ? 4 : 2), a_type == SK_A_FP32);
+  const bool tma_ok = tma_layout_ok(A, lda, a_type == SK_A_FP32 ? 4 : 2);
+  s = choose_tile(p, n, rows, di, &cfg, tma_ok, a_type);
   if (s != SK_OK) return s;
+  if (cfg.reg_tile && !totals_available(p, n, row_begin, row_end, R_fixed > 0 ? R_fixed : cfg.R, st)) {
+    s = choose_tile(p, n, rows, di, &cfg, tma_ok, a_type, false);
+    if (s != SK_OK) return s;
+  }
   if (cfg.own && a_type != SK_A_FP32) return set_error(SK_ERR_UNSUPPORTED, "the owner kernel reads FP32 A only");
   if (R_fixed > 0) cfg.R = R_fixed;
   TileLaunch L;
@@ -551,18 +572,9 @@ sk_status enqueue_sketch(sk_plan_s* p, const void* A, int64_t lda, int64_t n, in
   L.status = p->dstatus;
   L.P = nullptr;
   if (cfg.slices > 1 && cfg.long_slices == 1 && !cfg.glob && !cfg.reg) {
-    // One launch, as with one slice per chunk, which needs no chunk totals: taken where these would have
-    // to be allocated and the scratch limit or a stream capture forbids it.
-    L.fuse_finish = zero_y ? 1 : 0;
-    const size_t needP = sizeof(float) * (size_t)launch_P_floats(L);
-    if (p->tileP_bytes < needP) {
-      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-      const bool free = cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
-      if (!free || (p->scratch_limit > 0 &&
-                    plan_scratch_bytes(p) - p->tileP_bytes + needP > (size_t)p->scratch_limit))
-        L.slices = cfg.slices = 1;
-    }
-    if (cfg.slices == 1) L.fuse_finish = 0;
+    // One launch, as with one slice per chunk, which needs no chunk totals and is taken where these cannot be had.
+    if (totals_available(p, n, row_begin, row_end, cfg.R, st)) L.fuse_finish = zero_y ? 1 : 0;
+    else L.slices = cfg.slices = 1;
   }
   if (cfg.slices > 1 || cfg.glob || cfg.reg) {
     const size_t needP = sizeof(float) * (size_t)launch_P_floats(L);
@@ -1150,13 +1162,13 @@ sk_status sk_apply_partials(sk_plan p, const float* A, int64_t lda, int64_t n, f
   s = dev_info(&di);
   if (s != SK_OK) return s;
   TileCfg cfg;
-  s = choose_tile(p, n, p->m, di, &cfg, tma_layout_ok(A, lda), true);
+  s = choose_tile(p, n, p->m, di, &cfg, tma_layout_ok(A, lda));
   if (s != SK_OK) return s;
   if (cfg.glob) {
     // The global kernel finishes its passes as it goes; partials take the tile kernel instead.
     sk_plan_s tmp = *p;
     tmp.kernel = SK_KERNEL_TILE;
-    s = choose_tile(&tmp, n, p->m, di, &cfg, tma_layout_ok(A, lda), true);
+    s = choose_tile(&tmp, n, p->m, di, &cfg, tma_layout_ok(A, lda));
     if (s != SK_OK) return s;
   }
   cfg.R = R;
@@ -1304,7 +1316,7 @@ sk_status noalloc_tile_launch(const sk_plan_s* p, const float* A, int64_t lda, i
   s = dev_info(&di);
   if (s != SK_OK) return s;
   TileCfg cfg;
-  s = choose_tile(p, n, p->m, di, &cfg, tma_layout_ok(A, lda));
+  s = choose_tile(p, n, p->m, di, &cfg, tma_layout_ok(A, lda));  // FP32 A: never reg_tile
   if (s != SK_OK) return s;
   L->A = A;
   L->Y = Y;

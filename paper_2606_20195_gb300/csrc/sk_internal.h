@@ -33,7 +33,7 @@ struct TileLaunch {
   int32_t own = 0;    // 1: owner kernel (NC = 32, kb = 1 or 2 blocks per item, A through TMA)
   int32_t vec = 0;    // 1: n = 1 vector path of the tile kernel (NC = 4, no TMA)
   int32_t glob = 0;   // 1: global-accumulator kernel (chunk totals in P, any d); needs P
-  int32_t reg = 0;    // 1: register kernel (FP32 A through TMA, 32 columns x 1024 output rows per item); needs P
+  int32_t reg = 0;    // 1: register kernel (A through TMA; 32 columns x 1024 output rows per item, 16-bit A 64 x 512); needs P
   int32_t reg_nsub = 0, reg_cap = 0;  // register kernel: TMA copies per staged box, list entries per output row
   int32_t fuse_finish = 0;  // 1: tile kernel with slices > 1 as one cooperative launch that also writes all of Y
   int32_t no_finish = 0;  // 1: leave the chunk totals in P (no chunk-finish launch); P is then the caller's
@@ -64,20 +64,19 @@ void tile_geometry(const TileLaunch& L, int64_t* chunks, int32_t* ncg, int32_t* 
 // Passes of the global-accumulator kernel: column slabs of *ns columns and batches of *cb chunks,
 // chosen so that the chunk totals of one pass (cb x d x ns FP32) stay resident in L2.
 void global_passes(const TileLaunch& L, int64_t* ns, int64_t* cb);
+constexpr int64_t kBarrierFloats = 2;
 // FP32 elements of chunk-total scratch P a launch needs (0: none), with the barrier words of fuse_finish.
 int64_t launch_P_floats(const TileLaunch& L);
 // The global-accumulator kernel and its chunk finish, in passes (sk_global.cu); needs L.P.
 cudaError_t launch_global(const TileLaunch& L, cudaStream_t st, int32_t* launches);
-// Register kernel (sk_reg.cu): shared-memory bytes for a box of nsub TMA copies, lists of cap entries
-// and overflow lists of ovf_cap entries; threads per CTA; output rows per work item; blocks of S that
-// reach the widest group of output rows; the box and capacity for a sketch of d rows and block height
-// B within `smem_limit` bytes (cap_fixed > 0 imposes the capacity; false if nothing fits); and the
-// launch (its chunk finish included; needs L.P).
-size_t reg_smem_bytes(int32_t nsub, int32_t cap, int32_t ovf_cap);
-int32_t reg_threads();
-int32_t reg_targets();
-int32_t reg_blocks_per_group(int64_t d, int64_t B);
-bool reg_choose_box(int64_t d, int64_t B, size_t smem_limit, int32_t cap_fixed, int32_t* nsub, int32_t* cap);
+// Register kernel (sk_reg.cu): threads per CTA, output rows and columns per work item; the box and list
+// capacity for a sketch of d rows and block height B within `smem_limit` bytes (cap_fixed > 0 imposes the
+// capacity; false if nothing fits); and the launch (its chunk finish included; needs L.P).
+int32_t reg_threads(int32_t a_type);
+int32_t reg_targets(int32_t a_type);
+int32_t reg_cols(int32_t a_type);
+bool reg_choose_box(int64_t d, int64_t B, int32_t a_type, size_t smem_limit, int32_t cap_fixed, int32_t* nsub,
+                    int32_t* cap);
 cudaError_t launch_reg(const TileLaunch& L, cudaStream_t st, int32_t* launches);
 // Resident CTAs per SM of the tile kernel for (rule, threads, dynamic shared memory).
 int32_t tile_ctas_per_sm(int32_t rule, int32_t threads, size_t smem);

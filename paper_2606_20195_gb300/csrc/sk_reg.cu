@@ -36,6 +36,12 @@
 // produce), which the CTA's quarter-warps add into the chunk totals with FP32 vector reductions (one
 // 128-byte row per quarter-warp access). At the end of the item every thread adds its 32 sums into P.
 //
+// 16-bit A: a staged row of 128 bytes holds 64 columns, converted to FP32 as they are added. A thread then
+// keeps 64 sums, and the CTA has 512 threads and output rows: the same accumulators, boxes and row reads,
+// with a list entry and its 128 bytes serving twice the columns. At 2^22 x 64, d = 4096, k = 8, bfloat16:
+// 765 us, against 1332 us in the tile kernel, which is bound by its shared-memory additions whatever the
+// bytes of A.
+//
 // All rounding happens in the FP32 additions of the partial sums (any order within the chunk, as in
 // the tile kernel's atomic mode) and in the chunk finish; the result is the chunk total of the
 // canonical order up to the FP32 summation order inside the chunk.
@@ -52,10 +58,17 @@ namespace sk {
 
 namespace {
 
-constexpr int kRegThreads = 1024;
-constexpr int kRegTargets = kRegThreads;  // output rows per work item: one per thread
-constexpr int kRegCopyRows = 128;         // rows per TMA copy (16 KiB)
-constexpr int kRegMaxSub = 6;             // TMA copies per staged box (768 rows < kRegThreads: one row per thread)
+constexpr int kRegRowBytes = 128;  // a staged row: 32 FP32 or 64 16-bit columns
+constexpr int kRegCopyRows = 128;  // rows per TMA copy (16 KiB)
+constexpr int kRegMaxSub = 6;      // TMA copies per staged box (768 rows)
+
+// Columns per work item and threads (= output rows per work item) for the element type of A: the
+// accumulators take half of the register file either way.
+template <int AT>
+struct RegShape {
+  static constexpr int kCols = AT == kAF32 ? 32 : 64;
+  static constexpr int kThreads = AT == kAF32 ? 1024 : 512;
+};
 
 // A work item, written to shared memory by one thread (two descriptors: the current and the next item).
 struct RegItem {
@@ -67,10 +80,10 @@ struct RegItem {
 
 // Shared memory (byte offsets): two list-length arrays | 4 overflow counters (by box sequence mod 4) |
 // 2 mbarriers | 2 item descriptors (these at fixed offsets) | two staged boxes | two list tables
-// (kRegTargets x cap 16-bit entries, slot-major: [slot][output row]) | two overflow lists (ovf_cap
+// (threads x cap 16-bit entries, slot-major: [slot][output row]) | two overflow lists (ovf_cap
 // 32-bit entries: output row << 16 | row of the box | sign << 15).
 constexpr uint32_t kRegCnt = 0;
-constexpr uint32_t kRegNov = 2u * kRegTargets * 4u;
+constexpr uint32_t kRegNov = 2u * 1024u * 4u;
 constexpr uint32_t kRegBar = kRegNov + 16u;
 constexpr uint32_t kRegItem = kRegBar + 16u;
 constexpr uint32_t kRegStage = (kRegItem + 2u * (uint32_t)sizeof(RegItem) + 127u) & ~127u;
@@ -79,10 +92,10 @@ struct RegSmem {
   uint32_t tab, tab_stride, ovf, total;
 };
 
-__host__ __device__ inline RegSmem reg_smem(int32_t nsub, int32_t cap, int32_t ovf_cap) {
+__host__ __device__ inline RegSmem reg_smem(int32_t threads, int32_t nsub, int32_t cap, int32_t ovf_cap) {
   RegSmem L;
-  L.tab = kRegStage + 2u * (uint32_t)nsub * kRegCopyRows * 128u;
-  L.tab_stride = ((uint32_t)kRegTargets * (uint32_t)cap * 2u + 15u) & ~15u;
+  L.tab = kRegStage + 2u * (uint32_t)nsub * kRegCopyRows * kRegRowBytes;
+  L.tab_stride = ((uint32_t)threads * (uint32_t)cap * 2u + 15u) & ~15u;
   L.ovf = L.tab + 2u * L.tab_stride;
   L.total = L.ovf + 2u * (uint32_t)ovf_cap * 4u;
   return L;
@@ -117,6 +130,7 @@ __device__ __forceinline__ void red_quad(float* p, int64_t n, int64_t col0, floa
   }
 }
 
+template <int AT>
 __device__ __forceinline__ void reg_item(const RegGrid& G, int64_t w, int32_t rbox, RegItem* I) {
   const int32_t tg = (int32_t)(w % G.ntg);
   int64_t rest = w / G.ntg;
@@ -131,8 +145,8 @@ __device__ __forceinline__ void reg_item(const RegGrid& G, int64_t w, int32_t rb
   const int64_t r1 = c0 + (c1 - c0) * (sl + 1) / G.slices;
   const int64_t B = G.D.B;
   const int64_t d = B * G.D.k;
-  const int64_t tr0 = (int64_t)tg * kRegTargets;
-  const int64_t ntr = min((int64_t)kRegTargets, d - tr0);
+  const int64_t tr0 = (int64_t)tg * RegShape<AT>::kThreads;
+  const int64_t ntr = min((int64_t)RegShape<AT>::kThreads, d - tr0);
   I->r0 = r0;
   I->r1 = r1;
   I->tr0 = (int32_t)tr0;
@@ -142,45 +156,68 @@ __device__ __forceinline__ void reg_item(const RegGrid& G, int64_t w, int32_t rb
   I->plo = I->jlo >> 1;
   I->np = (I->jhi >> 1) - I->plo + 1;
   I->nbox = (int32_t)((r1 - r0 + rbox - 1) / rbox);
-  I->xcol = g * 32;
+  I->xcol = g * RegShape<AT>::kCols;
   I->ybase = (int32_t)(r0 - G.D.row_base);
   I->tl = (int32_t)tl;
 }
 
-// Step 1 for box b of the item (box sequence number seq): this thread's row (if the box has it) into
-// the lists of buffer seq & 1, or into the overflow list.
-template <int NSUB>
+// Step 1 for box b of the item (box sequence number seq): this thread's rows of the box (one, or up to
+// two with 512 threads) into the lists of buffer seq & 1, or into the overflow list.
+template <int NSUB, int AT>
 __device__ __forceinline__ void reg_hash(const RegGrid& G, const RegItem* I, int32_t b, uint32_t seq,
                                          unsigned char* sm) {
-  const int32_t tid = (int32_t)threadIdx.x;
+  constexpr uint32_t targets = RegShape<AT>::kThreads;
   constexpr int32_t rbox = NSUB * kRegCopyRows;
   const int64_t rb0 = I->r0 + (int64_t)b * rbox;
-  if ((int64_t)tid >= I->r1 - rb0 || tid >= rbox) return;
   uint16_t* tab = reinterpret_cast<uint16_t*>(sm + G.S.tab + (seq & 1u) * G.S.tab_stride);
-  uint32_t* cnt = reinterpret_cast<uint32_t*>(sm + kRegCnt) + (seq & 1u) * kRegTargets;
+  uint32_t* cnt = reinterpret_cast<uint32_t*>(sm + kRegCnt) + (seq & 1u) * targets;
   uint32_t* ovf = reinterpret_cast<uint32_t*>(sm + G.S.ovf) + (seq & 1u) * (uint32_t)G.ovf_cap;
   uint32_t* nov = reinterpret_cast<uint32_t*>(sm + kRegNov) + (seq & 3u);
   const uint32_t B = G.D.B;
   const int32_t np = I->np, plo = I->plo, jlo = I->jlo, jhi = I->jhi, tr0 = I->tr0;
   const uint32_t ntr = (uint32_t)I->ntr;
-  for (int32_t pr = 0; pr < np; ++pr) {
-    const uint32_t p = (uint32_t)(plo + pr);
-    const uint64_t h = row_pair_bits(G.D.seed, (uint64_t)(rb0 + tid), G.D.kp, p);
+  // (with at least as many threads as box rows this is one pass, and no loop)
+  for (int32_t i = (int32_t)threadIdx.x; i < rbox && i < I->r1 - rb0; i += targets) {
+    for (int32_t pr = 0; pr < np; ++pr) {
+      const uint32_t p = (uint32_t)(plo + pr);
+      const uint64_t h = row_pair_bits(G.D.seed, (uint64_t)(rb0 + i), G.D.kp, p);
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int32_t j = 2 * (int32_t)p + e;
-      if (j < jlo || j > jhi) continue;
-      const uint32_t wd = e ? (uint32_t)h : (uint32_t)(h >> 32);
-      const int32_t tgt = j * (int32_t)B + (int32_t)word_to_slot(wd, B) - tr0;  // d < 2^31
-      if ((uint32_t)tgt >= ntr) continue;
-      const uint32_t ent = (uint32_t)tid | ((wd & 1u) << 15);
-      const uint32_t pos = atomicAdd(cnt + tgt, 1u);
-      if (pos < (uint32_t)G.cap) {
-        tab[pos * kRegTargets + (uint32_t)tgt] = (uint16_t)ent;
-      } else {
-        const uint32_t o = atomicAdd(nov, 1u);
-        if (o < (uint32_t)G.ovf_cap) ovf[o] = ((uint32_t)tgt << 16) | ent;  // holds every entry of a box
+      for (int e = 0; e < 2; ++e) {
+        const int32_t j = 2 * (int32_t)p + e;
+        if (j < jlo || j > jhi) continue;
+        const uint32_t wd = e ? (uint32_t)h : (uint32_t)(h >> 32);
+        const int32_t tgt = j * (int32_t)B + (int32_t)word_to_slot(wd, B) - tr0;  // d < 2^31
+        if ((uint32_t)tgt >= ntr) continue;
+        const uint32_t ent = (uint32_t)i | ((wd & 1u) << 15);
+        const uint32_t pos = atomicAdd(cnt + tgt, 1u);
+        if (pos < (uint32_t)G.cap) {
+          tab[pos * targets + (uint32_t)tgt] = (uint16_t)ent;
+        } else {
+          const uint32_t o = atomicAdd(nov, 1u);
+          if (o < (uint32_t)G.ovf_cap) ovf[o] = ((uint32_t)tgt << 16) | ent;  // holds every entry of a box
+        }
       }
+    }
+    if (rbox <= (int32_t)targets) break;
+  }
+}
+
+// The FP32 values of 16 bytes of A, as pairs, added with the sign to a chunk's sums.
+template <int AT>
+__device__ __forceinline__ void reg_add(const uint4& v, float sg, float2* a) {
+  const float2 s2 = make_float2(sg, sg);
+  const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+  if constexpr (AT == kAF32) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      a[h] = __ffma2_rn(make_float2(__uint_as_float(u[2 * h]), __uint_as_float(u[2 * h + 1])), s2, a[h]);
+  } else {
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      float2 f;
+      if constexpr (AT == kABF16) f = make_float2(__uint_as_float(u[h] << 16), __uint_as_float(u[h] & 0xFFFF0000u));
+      else f = __half22float2(*reinterpret_cast<const __half2*>(&u[h]));
+      a[h] = __ffma2_rn(f, s2, a[h]);
     }
   }
 }
@@ -191,28 +228,30 @@ __device__ __forceinline__ void reg_hash(const RegGrid& G, const RegItem* I, int
 template <int NSUB>
 __device__ __forceinline__ void reg_issue_box(const CUtensorMap* tmap, const RegItem* I, int32_t b, int32_t buf,
                                               unsigned char* sm) {
-  constexpr uint32_t box_bytes = (uint32_t)NSUB * kRegCopyRows * 128u;
+  constexpr uint32_t box_bytes = (uint32_t)NSUB * kRegCopyRows * kRegRowBytes;
   uint64_t* bar = reinterpret_cast<uint64_t*>(sm + kRegBar) + buf;
   fence_proxy_async_smem();
   mbar_arrive_expect_tx(bar, box_bytes);
 #pragma unroll
   for (int c = 0; c < NSUB; ++c)
-    tma_load_2d(sm + kRegStage + (size_t)buf * box_bytes + (size_t)c * kRegCopyRows * 128, tmap, I->xcol,
+    tma_load_2d(sm + kRegStage + (size_t)buf * box_bytes + (size_t)c * kRegCopyRows * kRegRowBytes, tmap, I->xcol,
                 I->ybase + (b * NSUB + c) * kRegCopyRows, bar);
 }
 
 // NSUB: TMA copies per staged box (box = NSUB * 128 rows), a compile-time constant so that the box
 // layout and the copy issue (on every box's critical path) are fixed.
-template <int NSUB>
-__global__ void __launch_bounds__(kRegThreads, 1) reg_kernel(const RegGrid G, const __grid_constant__ CUtensorMap tmap) {
+template <int NSUB, int AT>
+__global__ void __launch_bounds__(RegShape<AT>::kThreads, 1) reg_kernel(const RegGrid G, const __grid_constant__ CUtensorMap tmap) {
+  constexpr int threads = RegShape<AT>::kThreads;
+  constexpr int kPairs = RegShape<AT>::kCols / 16;  // FP32 pairs per 16-byte chunk of a row
   extern __shared__ __align__(128) unsigned char sm[];
   const int tid = threadIdx.x;
-  if (blockDim.x != kRegThreads || G.nsub != NSUB || G.cap < 1 || G.ovf_cap < 0) {
+  if (blockDim.x != threads || G.nsub != NSUB || G.cap < 1 || G.ovf_cap < 0) {
     if (tid == 0 && G.status) atomicOr(G.status, kStatusBounds);
     return;
   }
   constexpr int32_t rbox = NSUB * kRegCopyRows;
-  constexpr uint32_t box_bytes = (uint32_t)rbox * 128u;
+  constexpr uint32_t box_bytes = (uint32_t)rbox * kRegRowBytes;
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kRegBar);
   RegItem* items = reinterpret_cast<RegItem*>(sm + kRegItem);
   uint32_t* nov = reinterpret_cast<uint32_t*>(sm + kRegNov);
@@ -220,19 +259,21 @@ __global__ void __launch_bounds__(kRegThreads, 1) reg_kernel(const RegGrid G, co
     mbar_init(bars, 1);
     mbar_init(bars + 1, 1);
     mbar_fence_init();
-    reg_item(G, blockIdx.x, rbox, items);
+    reg_item<AT>(G, blockIdx.x, rbox, items);
   }
   if (tid < 4) nov[tid] = 0u;
   reinterpret_cast<uint32_t*>(sm + kRegCnt)[tid] = 0u;
-  reinterpret_cast<uint32_t*>(sm + kRegCnt)[kRegTargets + tid] = 0u;
+  reinterpret_cast<uint32_t*>(sm + kRegCnt)[threads + tid] = 0u;
   const uint32_t l16 = (uint32_t)(tid & 7) << 4;  // this lane's chunk rotation (bytes), lane mod 8
   // Bit b of `par`: parity of the next phase of buffer b's mbarrier (toggled after every wait; in
   // thread 0 only after a wait that succeeded). Bit b of `pend` (thread 0): a box copied into buffer b
   // has not been seen complete yet. `sq`: boxes this CTA has started (picks list buffers and counters).
   uint32_t par = 0u, pend = 0u, sq = 0u, cur = 0u;
-  float2 acc[8][2];
+  float2 acc[8][kPairs];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) acc[q][0] = acc[q][1] = make_float2(0.f, 0.f);
+  for (int q = 0; q < 8; ++q)
+#pragma unroll
+    for (int h = 0; h < kPairs; ++h) acc[q][h] = make_float2(0.f, 0.f);
   bool aborted = false;
   for (int64_t w = blockIdx.x; w < G.items; w += gridDim.x, cur ^= 1u) {
     __syncthreads();  // this item's descriptor is written; the last item's readers of the other are done
@@ -243,19 +284,19 @@ __global__ void __launch_bounds__(kRegThreads, 1) reg_kernel(const RegGrid G, co
         pend |= 1u << b;
       }
     }
-    if (tid == 32 && w + gridDim.x < G.items) reg_item(G, w + gridDim.x, rbox, items + (cur ^ 1u));
-    reg_hash<NSUB>(G, I, 0, sq, sm);
+    if (tid == 32 && w + gridDim.x < G.items) reg_item<AT>(G, w + gridDim.x, rbox, items + (cur ^ 1u));
+    reg_hash<NSUB, AT>(G, I, 0, sq, sm);
     __syncthreads();
     const int32_t nbox = I->nbox;
     for (int32_t b = 0; b < nbox; ++b, ++sq) {
       const int buf = b & 1;
       // 1. Hash the next box (its lists are the other buffer, emptied a box ago).
-      if (b + 1 < nbox) reg_hash<NSUB>(G, I, b + 1, sq + 1u, sm);
+      if (b + 1 < nbox) reg_hash<NSUB, AT>(G, I, b + 1, sq + 1u, sm);
       const bool ok = mbar_wait_bounded(bars + buf, (par >> buf) & 1u);
       if (ok || tid != 0) par ^= 1u << buf;
       if (tid == 0 && ok) pend &= ~(1u << buf);
       const unsigned char* st = sm + kRegStage + (size_t)buf * box_bytes;
-      uint32_t* cn = reinterpret_cast<uint32_t*>(sm + kRegCnt) + (sq & 1u) * kRegTargets;
+      uint32_t* cn = reinterpret_cast<uint32_t*>(sm + kRegCnt) + (sq & 1u) * threads;
       if (ok) {
         // 2a. Overflow rows, one per quarter-warp: 8 lanes read the row's 128 bytes and reduce them
         //     into the chunk totals of their output row.
@@ -263,28 +304,29 @@ __global__ void __launch_bounds__(kRegThreads, 1) reg_kernel(const RegGrid G, co
         const uint32_t* ov = reinterpret_cast<const uint32_t*>(sm + G.S.ovf) + (sq & 1u) * (uint32_t)G.ovf_cap;
         const int ql = tid & 7;
         const int64_t n = G.D.n;
-        const int64_t col0 = (int64_t)I->xcol + 4 * ql;
-        for (uint32_t o = (uint32_t)(tid >> 3); o < no; o += kRegThreads / 8) {
+        const int64_t col0 = (int64_t)I->xcol + (2 * kPairs) * ql;
+        for (uint32_t o = (uint32_t)(tid >> 3); o < no; o += threads / 8) {
           const uint32_t e = ov[o];
-          float4 v = *reinterpret_cast<const float4*>(st + ((e & 0x7FFFu) << 7) + ql * 16);
-          if (e & 0x8000u) v = make_float4(-v.x, -v.y, -v.z, -v.w);
-          float* Pt = G.P + (int64_t)I->tl * ((int64_t)G.D.B * G.D.k * n);
-          if (col0 < n) red_quad(Pt + ((int64_t)I->tr0 + (e >> 16)) * n + col0, n, col0, v);
+          float2 v[kPairs];
+#pragma unroll
+          for (int h = 0; h < kPairs; ++h) v[h] = make_float2(0.f, 0.f);
+          reg_add<AT>(*reinterpret_cast<const uint4*>(st + ((e & 0x7FFFu) << 7) + ql * 16), (e & 0x8000u) ? -1.f : 1.f, v);
+          float* Pt = G.P + (int64_t)I->tl * ((int64_t)G.D.B * G.D.k * n) + ((int64_t)I->tr0 + (e >> 16)) * n;
+#pragma unroll
+          for (int h = 0; h < kPairs; h += 2)
+            if (col0 + 2 * h < n)
+              red_quad(Pt + col0 + 2 * h, n, col0 + 2 * h, make_float4(v[h].x, v[h].y, v[h + 1].x, v[h + 1].y));
         }
         // 2b. This thread's list.
         const uint16_t* tb = reinterpret_cast<const uint16_t*>(sm + G.S.tab + (sq & 1u) * G.S.tab_stride);
         const uint32_t ns = min(cn[tid], (uint32_t)G.cap);
         for (uint32_t i = 0; i < ns; ++i) {
-          const uint32_t e = tb[i * kRegTargets + tid];
+          const uint32_t e = tb[i * threads + tid];
           const uint32_t ra = ((e & 0x7FFFu) << 7) | l16;
           const float sg = __uint_as_float(((e & 0x8000u) << 16) | 0x3F800000u);
-          const float2 s2 = make_float2(sg, sg);
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const float4 v = *reinterpret_cast<const float4*>(st + (ra ^ ((uint32_t)q << 4)));
-            acc[q][0] = __ffma2_rn(make_float2(v.x, v.y), s2, acc[q][0]);
-            acc[q][1] = __ffma2_rn(make_float2(v.z, v.w), s2, acc[q][1]);
-          }
+          for (int q = 0; q < 8; ++q)
+            reg_add<AT>(*reinterpret_cast<const uint4*>(st + (ra ^ ((uint32_t)q << 4))), sg, acc[q]);
         }
         cn[tid] = 0u;
       }
@@ -306,13 +348,19 @@ __global__ void __launch_bounds__(kRegThreads, 1) reg_kernel(const RegGrid G, co
       const int64_t xcol = I->xcol;
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        const int64_t col0 = xcol + (int64_t)(((uint32_t)q << 2) ^ (l16 >> 2));
-        const float4 v = make_float4(acc[q][0].x, acc[q][0].y, acc[q][1].x, acc[q][1].y);
-        if (col0 < n && (v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f)) red_quad(prow + col0, n, col0, v);
+        const int64_t col0 = xcol + (int64_t)((((uint32_t)q << 4) ^ l16) >> 4) * (2 * kPairs);
+#pragma unroll
+        for (int h = 0; h < kPairs; h += 2) {
+          const float4 v = make_float4(acc[q][h].x, acc[q][h].y, acc[q][h + 1].x, acc[q][h + 1].y);
+          if (col0 + 2 * h < n && (v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f))
+            red_quad(prow + col0 + 2 * h, n, col0 + 2 * h, v);
+        }
       }
     }
 #pragma unroll
-    for (int q = 0; q < 8; ++q) acc[q][0] = acc[q][1] = make_float2(0.f, 0.f);
+    for (int q = 0; q < 8; ++q)
+#pragma unroll
+      for (int h = 0; h < kPairs; ++h) acc[q][h] = make_float2(0.f, 0.f);
   }
   if (aborted && tid == 0) {
     if (G.status) atomicOr(G.status, kStatusTimeout);
@@ -323,23 +371,37 @@ __global__ void __launch_bounds__(kRegThreads, 1) reg_kernel(const RegGrid G, co
   }
 }
 
+using RegKernelFn = void (*)(const RegGrid, const CUtensorMap);
+
+template <int AT>
+RegKernelFn reg_kernel_for(int32_t nsub) {
+  switch (nsub) {
+    case 1: return reg_kernel<1, AT>;
+    case 2: return reg_kernel<2, AT>;
+    case 3: return reg_kernel<3, AT>;
+    case 4: return reg_kernel<4, AT>;
+    case 5: return reg_kernel<5, AT>;
+    default: return reg_kernel<6, AT>;
+  }
+}
+
 }  // namespace
 
-size_t reg_smem_bytes(int32_t nsub, int32_t cap, int32_t ovf_cap) { return reg_smem(nsub, cap, ovf_cap).total; }
+int32_t reg_threads(int32_t a_type) { return a_type == kAF32 ? RegShape<kAF32>::kThreads : RegShape<kABF16>::kThreads; }
+
+int32_t reg_targets(int32_t a_type) { return reg_threads(a_type); }
+
+int32_t reg_cols(int32_t a_type) { return a_type == kAF32 ? RegShape<kAF32>::kCols : RegShape<kABF16>::kCols; }
 
 // Blocks of S that reach the widest target group of a sketch with d rows and block height B.
-int32_t reg_blocks_per_group(int64_t d, int64_t B) {
+static int32_t reg_blocks_per_group(int64_t d, int64_t B, int32_t targets) {
   int32_t nbg = 1;
-  for (int64_t tr0 = 0; tr0 < d; tr0 += kRegTargets) {
-    const int64_t tr1 = std::min<int64_t>(d, tr0 + kRegTargets) - 1;
+  for (int64_t tr0 = 0; tr0 < d; tr0 += targets) {
+    const int64_t tr1 = std::min<int64_t>(d, tr0 + targets) - 1;
     nbg = std::max<int32_t>(nbg, (int32_t)(tr1 / B - tr0 / B + 1));
   }
   return nbg;
 }
-
-int32_t reg_threads() { return kRegThreads; }
-
-int32_t reg_targets() { return kRegTargets; }
 
 // List capacity for lambda entries per output row and box (a Poisson mean): about
 // lambda + 1.5 sqrt(lambda), at least 2. A thread's list costs as many steps as the longest list of its
@@ -354,12 +416,13 @@ static int32_t list_cap(double lam) {
 // capacity from list_cap for lambda = box rows / B, or cap_fixed if positive. The overflow list holds
 // every entry a box can produce (box rows x blocks reaching a target group), so no entry is ever
 // dropped. False if nothing fits.
-bool reg_choose_box(int64_t d, int64_t B, size_t smem_limit, int32_t cap_fixed, int32_t* nsub, int32_t* cap) {
-  const int32_t nbg = reg_blocks_per_group(d, B);
+bool reg_choose_box(int64_t d, int64_t B, int32_t a_type, size_t smem_limit, int32_t cap_fixed, int32_t* nsub,
+                    int32_t* cap) {
+  const int32_t nbg = reg_blocks_per_group(d, B, reg_targets(a_type));
   for (int32_t s = kRegMaxSub; s >= 1; --s) {
     const double lam = (double)(s * kRegCopyRows) / (double)std::max<int64_t>(B, 1);
     const int32_t c = cap_fixed > 0 ? cap_fixed : list_cap(lam);
-    if (reg_smem(s, c, s * kRegCopyRows * nbg).total <= smem_limit) {
+    if (reg_smem(reg_threads(a_type), s, c, s * kRegCopyRows * nbg).total <= smem_limit) {
       *nsub = s;
       *cap = c;
       return true;
@@ -369,7 +432,7 @@ bool reg_choose_box(int64_t d, int64_t B, size_t smem_limit, int32_t cap_fixed, 
 }
 
 cudaError_t launch_reg(const TileLaunch& L, cudaStream_t st, int32_t* launches) {
-  if (L.a_type != kAF32 || !L.P || L.reg_nsub < 1 || L.reg_nsub > kRegMaxSub || L.reg_cap < 1)
+  if (!L.P || L.reg_nsub < 1 || L.reg_nsub > kRegMaxSub || L.reg_cap < 1)
     return cudaErrorInvalidValue;
   RegGrid G;
   memset(&G, 0, sizeof(G));
@@ -384,18 +447,19 @@ cudaError_t launch_reg(const TileLaunch& L, cudaStream_t st, int32_t* launches) 
   G.D.B = (uint32_t)B;
   G.D.k = (uint32_t)L.k;
   G.D.kp = (uint32_t)((L.k + 1) / 2);
-  G.D.log2NC = 5;
+  G.D.log2NC = L.a_type == kAF32 ? 5 : 6;
   G.D.S = 1;
   G.D.kb = L.k;
   G.D.col_off = L.col_off;
-  G.D.a_type = kAF32;
+  G.D.a_type = L.a_type;
   G.row_begin = L.row_begin;
   G.row_end = L.row_end;
   G.R = L.R;
   G.t_first = L.row_begin / L.R;
   const int64_t chunks = (L.row_end - 1) / L.R - G.t_first + 1;
-  G.ncg = (int32_t)((L.n + 31) / 32);
-  G.ntg = (int32_t)((L.d + kRegTargets - 1) / kRegTargets);
+  const int32_t cols = reg_cols(L.a_type), targets = reg_targets(L.a_type), threads = reg_threads(L.a_type);
+  G.ncg = (int32_t)((L.n + cols - 1) / cols);
+  G.ntg = (int32_t)((L.d + targets - 1) / targets);
   G.slices = std::max(1, L.slices);
   G.items = chunks * G.slices * G.ncg * G.ntg;
   G.nsub = L.reg_nsub;
@@ -407,27 +471,21 @@ cudaError_t launch_reg(const TileLaunch& L, cudaStream_t st, int32_t* launches) 
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  G.ovf_cap = G.nsub * kRegCopyRows * reg_blocks_per_group(L.d, B);  // every entry of a box
-  G.S = reg_smem(G.nsub, G.cap, G.ovf_cap);
+  G.ovf_cap = G.nsub * kRegCopyRows * reg_blocks_per_group(L.d, B, targets);  // every entry of a box
+  G.S = reg_smem(threads, G.nsub, G.cap, G.ovf_cap);
   CUtensorMap tmap;
   memset(&tmap, 0, sizeof(tmap));
-  if (!encode_a_map(&tmap, L.A, kAF32, L.lda, L.n, L.row_end - L.row_begin, 32, kRegCopyRows))
+  if (!encode_a_map(&tmap, L.A, L.a_type, L.lda, L.n, L.row_end - L.row_begin, cols, kRegCopyRows))
     return cudaErrorInvalidValue;
   const size_t smem = G.S.total;
-  void (*kern)(const RegGrid, const CUtensorMap) = nullptr;
-  switch (G.nsub) {
-    case 1: kern = reg_kernel<1>; break;
-    case 2: kern = reg_kernel<2>; break;
-    case 3: kern = reg_kernel<3>; break;
-    case 4: kern = reg_kernel<4>; break;
-    case 5: kern = reg_kernel<5>; break;
-    default: kern = reg_kernel<6>; break;
-  }
+  const RegKernelFn kern = L.a_type == kAF16    ? reg_kernel_for<kAF16>(G.nsub)
+                           : L.a_type == kABF16 ? reg_kernel_for<kABF16>(G.nsub)
+                                                : reg_kernel_for<kAF32>(G.nsub);
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int64_t grid = L.grid > 0 ? L.grid : (int64_t)sms;
   grid = std::max<int64_t>(1, std::min<int64_t>(grid, G.items));
-  kern<<<(unsigned)grid, kRegThreads, smem, st>>>(G, tmap);
+  kern<<<(unsigned)grid, (unsigned)threads, smem, st>>>(G, tmap);
   if (launches) *launches += 1;
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
