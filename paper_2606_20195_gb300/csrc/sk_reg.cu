@@ -39,7 +39,7 @@
 // 16-bit A: a staged row of 128 bytes holds 64 columns, converted to FP32 as they are added. A thread then
 // keeps 64 sums, and the CTA has 512 threads and output rows: the same accumulators, boxes and row reads,
 // with a list entry and its 128 bytes serving twice the columns. At 2^22 x 64, d = 4096, k = 8, bfloat16:
-// 765 us, against 1332 us in the tile kernel, which is bound by its shared-memory additions whatever the
+// 732 us, against 1332 us in the tile kernel, which is bound by its shared-memory additions whatever the
 // bytes of A.
 //
 // All rounding happens in the FP32 additions of the partial sums (any order within the chunk, as in
@@ -75,7 +75,10 @@ struct RegItem {
   int64_t r0, r1;                 // global rows
   int32_t tr0, ntr;               // first output row of the group, output rows in it
   int32_t jlo, jhi, plo, np;      // blocks that reach the group, and their 64-bit stream outputs
-  int32_t nbox, xcol, ybase, tl;  // boxes, first column, row of A of r0, chunk index (from t_first)
+  int32_t nbox, xcol, ybase;      // boxes, first column, row of A of r0
+  int32_t cols;                   // columns of A from xcol on
+  uint64_t z0;                    // SplitMix64 state of row r0's first stream output for the group
+  float* P;                       // chunk totals at (tr0, xcol)
 };
 
 // Shared memory (byte offsets): two list-length arrays | 4 overflow counters (by box sequence mod 4) |
@@ -158,7 +161,9 @@ __device__ __forceinline__ void reg_item(const RegGrid& G, int64_t w, int32_t rb
   I->nbox = (int32_t)((r1 - r0 + rbox - 1) / rbox);
   I->xcol = g * RegShape<AT>::kCols;
   I->ybase = (int32_t)(r0 - G.D.row_base);
-  I->tl = (int32_t)tl;
+  I->cols = (int32_t)(G.D.n - I->xcol);
+  I->z0 = G.D.seed + ((uint64_t)r0 * G.D.kp + (uint32_t)I->plo + 1ull) * kSplitMixGamma;
+  I->P = G.P + tl * (d * G.D.n) + tr0 * G.D.n + I->xcol;
 }
 
 // Step 1 for box b of the item (box sequence number seq): this thread's rows of the box (one, or up to
@@ -175,12 +180,15 @@ __device__ __forceinline__ void reg_hash(const RegGrid& G, const RegItem* I, int
   uint32_t* nov = reinterpret_cast<uint32_t*>(sm + kRegNov) + (seq & 3u);
   const uint32_t B = G.D.B;
   const int32_t np = I->np, plo = I->plo, jlo = I->jlo, jhi = I->jhi, tr0 = I->tr0;
+  const int32_t left = (int32_t)min((int64_t)rbox, I->r1 - rb0);
   const uint32_t ntr = (uint32_t)I->ntr;
   // (with at least as many threads as box rows this is one pass, and no loop)
-  for (int32_t i = (int32_t)threadIdx.x; i < rbox && i < I->r1 - rb0; i += targets) {
-    for (int32_t pr = 0; pr < np; ++pr) {
+  for (int32_t i = (int32_t)threadIdx.x; i < left; i += targets) {
+    // state of row r0 + b * rbox + i: each row advances the stream by kp outputs
+    uint64_t z = I->z0 + (uint64_t)((uint32_t)(b * rbox + i)) * (G.D.kp * kSplitMixGamma);
+    for (int32_t pr = 0; pr < np; ++pr, z += kSplitMixGamma) {
       const uint32_t p = (uint32_t)(plo + pr);
-      const uint64_t h = row_pair_bits(G.D.seed, (uint64_t)(rb0 + i), G.D.kp, p);
+      const uint64_t h = splitmix_finalize(z);
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         const int32_t j = 2 * (int32_t)p + e;
@@ -264,6 +272,7 @@ __global__ void __launch_bounds__(RegShape<AT>::kThreads, 1) reg_kernel(const Re
   if (tid < 4) nov[tid] = 0u;
   reinterpret_cast<uint32_t*>(sm + kRegCnt)[tid] = 0u;
   reinterpret_cast<uint32_t*>(sm + kRegCnt)[threads + tid] = 0u;
+  const uint32_t sm32 = smem_addr(sm);
   const uint32_t l16 = (uint32_t)(tid & 7) << 4;  // this lane's chunk rotation (bytes), lane mod 8
   // Bit b of `par`: parity of the next phase of buffer b's mbarrier (toggled after every wait; in
   // thread 0 only after a wait that succeeded). Bit b of `pend` (thread 0): a box copied into buffer b
@@ -303,30 +312,39 @@ __global__ void __launch_bounds__(RegShape<AT>::kThreads, 1) reg_kernel(const Re
         const uint32_t no = min(nov[sq & 3u], (uint32_t)G.ovf_cap);
         const uint32_t* ov = reinterpret_cast<const uint32_t*>(sm + G.S.ovf) + (sq & 1u) * (uint32_t)G.ovf_cap;
         const int ql = tid & 7;
-        const int64_t n = G.D.n;
-        const int64_t col0 = (int64_t)I->xcol + (2 * kPairs) * ql;
+        const int32_t col0 = (2 * kPairs) * ql;
         for (uint32_t o = (uint32_t)(tid >> 3); o < no; o += threads / 8) {
           const uint32_t e = ov[o];
           float2 v[kPairs];
 #pragma unroll
           for (int h = 0; h < kPairs; ++h) v[h] = make_float2(0.f, 0.f);
           reg_add<AT>(*reinterpret_cast<const uint4*>(st + ((e & 0x7FFFu) << 7) + ql * 16), (e & 0x8000u) ? -1.f : 1.f, v);
-          float* Pt = G.P + (int64_t)I->tl * ((int64_t)G.D.B * G.D.k * n) + ((int64_t)I->tr0 + (e >> 16)) * n;
+          float* Pt = I->P + (int64_t)(e >> 16) * G.D.n + col0;
 #pragma unroll
           for (int h = 0; h < kPairs; h += 2)
-            if (col0 + 2 * h < n)
-              red_quad(Pt + col0 + 2 * h, n, col0 + 2 * h, make_float4(v[h].x, v[h].y, v[h + 1].x, v[h + 1].y));
+            if (col0 + 2 * h < I->cols)
+              red_quad(Pt + 2 * h, G.D.n, I->xcol + col0 + 2 * h, make_float4(v[h].x, v[h].y, v[h + 1].x, v[h + 1].y));
         }
         // 2b. This thread's list.
-        const uint16_t* tb = reinterpret_cast<const uint16_t*>(sm + G.S.tab + (sq & 1u) * G.S.tab_stride);
+        // (32-bit shared addresses: the XOR acts on the whole address, as a staged row is 128-byte aligned)
         const uint32_t ns = min(cn[tid], (uint32_t)G.cap);
-        for (uint32_t i = 0; i < ns; ++i) {
-          const uint32_t e = tb[i * threads + tid];
-          const uint32_t ra = ((e & 0x7FFFu) << 7) | l16;
-          const float sg = __uint_as_float(((e & 0x8000u) << 16) | 0x3F800000u);
+        uint32_t la = sm32 + G.S.tab + (sq & 1u) * G.S.tab_stride + 2u * (uint32_t)tid;
+        const uint32_t le = la + ns * (2u * threads);
+        const uint32_t rows = sm32 + kRegStage + (uint32_t)buf * box_bytes + l16;
+#pragma unroll 1
+        for (; la != le; la += 2u * threads) {
+          int32_t e;  // sign-extended: the sign of the entry is the sign of the register
+          asm volatile("ld.shared.s16 %0, [%1];" : "=r"(e) : "r"(la));
+          const uint32_t ra = rows + (((uint32_t)e & 0x7FFFu) << 7);
+          const float sg = __uint_as_float(((uint32_t)e & 0x80000000u) | 0x3F800000u);
 #pragma unroll
-          for (int q = 0; q < 8; ++q)
-            reg_add<AT>(*reinterpret_cast<const uint4*>(st + (ra ^ ((uint32_t)q << 4))), sg, acc[q]);
+          for (int q = 0; q < 8; ++q) {
+            uint4 v;
+            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                         : "r"(ra ^ ((uint32_t)q << 4)));
+            reg_add<AT>(v, sg, acc[q]);
+          }
         }
         cn[tid] = 0u;
       }
@@ -343,17 +361,15 @@ __global__ void __launch_bounds__(RegShape<AT>::kThreads, 1) reg_kernel(const Re
     if (aborted) break;
     // 3. The item's partial sums into the chunk totals (zero sums add nothing).
     if (tid < I->ntr) {
-      const int64_t n = G.D.n;
-      float* prow = G.P + (int64_t)I->tl * ((int64_t)G.D.B * G.D.k * n) + ((int64_t)I->tr0 + tid) * n;
-      const int64_t xcol = I->xcol;
+      float* prow = I->P + (int64_t)tid * G.D.n;
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        const int64_t col0 = xcol + (int64_t)((((uint32_t)q << 4) ^ l16) >> 4) * (2 * kPairs);
+        const int32_t col0 = (int32_t)((((uint32_t)q << 4) ^ l16) >> 4) * (2 * kPairs);
 #pragma unroll
         for (int h = 0; h < kPairs; h += 2) {
           const float4 v = make_float4(acc[q][h].x, acc[q][h].y, acc[q][h + 1].x, acc[q][h + 1].y);
-          if (col0 + 2 * h < n && (v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f))
-            red_quad(prow + col0 + 2 * h, n, col0 + 2 * h, v);
+          if (col0 + 2 * h < I->cols && (v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f))
+            red_quad(prow + col0 + 2 * h, G.D.n, I->xcol + col0 + 2 * h, v);
         }
       }
     }
