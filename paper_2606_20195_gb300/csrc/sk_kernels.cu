@@ -14,13 +14,14 @@
 
 namespace sk {
 
+template <bool FINISH>
 static TileKernelFn tile_kernel_f32(int32_t rule) {
   switch (rule) {
-    case kRN: return tile_kernel<kRN, float>;
-    case kSR: return tile_kernel<kSR, float>;
-    case kDither: return tile_kernel<kDither, float>;
-    case kBF16: return tile_kernel<kBF16, float>;
-    default: return tile_kernel<kFP32, float>;
+    case kRN: return tile_kernel<kRN, float, FINISH>;
+    case kSR: return tile_kernel<kSR, float, FINISH>;
+    case kDither: return tile_kernel<kDither, float, FINISH>;
+    case kBF16: return tile_kernel<kBF16, float, FINISH>;
+    default: return tile_kernel<kFP32, float, FINISH>;
   }
 }
 
@@ -141,7 +142,10 @@ cudaError_t launch_tile(const TileLaunch& L, cudaStream_t st, int32_t* launches)
   int sms = 0;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const TileKernelFn kern = (L.a_type == kAF32) ? tile_kernel_f32(L.rule) : tile_kernel_a16(L.rule, L.a_type);
+  const bool finish = L.fuse_finish && P.slices > 1;
+  const TileKernelFn kern = L.a_type != kAF32 ? tile_kernel_a16(L.rule, L.a_type, finish)
+                            : finish            ? tile_kernel_f32<true>(L.rule)
+                                                : tile_kernel_f32<false>(L.rule);
   if (!kern) return cudaErrorInvalidValue;
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -152,7 +156,7 @@ cudaError_t launch_tile(const TileLaunch& L, cudaStream_t st, int32_t* launches)
   int64_t grid = L.grid > 0 ? L.grid : (int64_t)sms * per_sm;
   grid = std::min<int64_t>(grid, P.items);
   if (grid < 1) grid = 1;
-  if (L.fuse_finish && P.slices > 1) {
+  if (finish) {
     P.bar = reinterpret_cast<unsigned*>(L.P + chunks * L.d * L.n);
     void* args[2] = {&P, &tmap};
     e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kern), dim3((unsigned)grid), dim3(L.threads), args,
@@ -187,7 +191,7 @@ template <int RULE>
 static void chunk_finish_launch(const TileDesc& D, float* P, int64_t t_first, int64_t chunks, cudaStream_t st) {
   const int64_t quads = (int64_t)D.B * D.k * ((D.n + 3) >> 2);
   const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((quads + 255) / 256, 1 << 16));
-  if (quads <= 65536) chunk_finish_kernel<RULE, 4><<<grid, 256, 0, st>>>(D, P, t_first, chunks);
+  if (quads <= 65536 && D.n % 4 == 0) chunk_finish_kernel<RULE, 4><<<grid, 256, 0, st>>>(D, P, t_first, chunks);
   else chunk_finish_kernel<RULE, 1><<<grid, 256, 0, st>>>(D, P, t_first, chunks);
 }
 
@@ -205,7 +209,7 @@ cudaError_t launch_chunk_finish(const TileDesc& D, int32_t rule, float* P, int64
 }
 
 int32_t tile_ctas_per_sm(int32_t rule, int32_t threads, size_t smem) {
-  const TileKernelFn kern = tile_kernel_f32(rule);
+  const TileKernelFn kern = tile_kernel_f32<false>(rule);
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;

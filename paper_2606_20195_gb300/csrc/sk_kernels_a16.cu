@@ -10,20 +10,20 @@
 
 namespace sk {
 
-template <typename TA>
+template <typename TA, bool FINISH>
 static TileKernelFn pick(int32_t rule) {
   switch (rule) {
-    case kRN: return tile_kernel<kRN, TA>;
-    case kSR: return tile_kernel<kSR, TA>;
-    case kDither: return tile_kernel<kDither, TA>;
-    case kBF16: return tile_kernel<kBF16, TA>;
-    default: return tile_kernel<kFP32, TA>;
+    case kRN: return tile_kernel<kRN, TA, FINISH>;
+    case kSR: return tile_kernel<kSR, TA, FINISH>;
+    case kDither: return tile_kernel<kDither, TA, FINISH>;
+    case kBF16: return tile_kernel<kBF16, TA, FINISH>;
+    default: return tile_kernel<kFP32, TA, FINISH>;
   }
 }
 
-TileKernelFn tile_kernel_a16(int32_t rule, int32_t a_type) {
-  if (a_type == kAF16) return pick<__half>(rule);
-  if (a_type == kABF16) return pick<__nv_bfloat16>(rule);
+TileKernelFn tile_kernel_a16(int32_t rule, int32_t a_type, bool finish) {
+  if (a_type == kAF16) return finish ? pick<__half, true>(rule) : pick<__half, false>(rule);
+  if (a_type == kABF16) return finish ? pick<__nv_bfloat16, true>(rule) : pick<__nv_bfloat16, false>(rule);
   return nullptr;
 }
 

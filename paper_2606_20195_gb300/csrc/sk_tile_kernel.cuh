@@ -40,7 +40,7 @@ __device__ __forceinline__ bool tile_grid_barrier(unsigned* bar, unsigned* statu
 // One CTA per SM (or per work item), work items in a grid-stride loop: scatter, then flush into Y or
 // into the chunk totals. TA is the element type of A; the FP32 instantiations live in sk_kernels.cu,
 // the 16-bit ones in sk_kernels_a16.cu (compiled in parallel).
-template <int RULE, typename TA>
+template <int RULE, typename TA, bool FINISH>
 __global__ void __launch_bounds__(1024) tile_kernel(const TileGrid P, const __grid_constant__ CUtensorMap tmap) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ int abort_flag;
@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(1024) tile_kernel(const TileGrid P, const __gr
     if (P.slices == 1) {
       tile_flush<RULE>(D, t, g, j0, kbe, acc);
     } else {
-      // slice partials into the chunk totals; the end of this kernel (P.bar) or chunk_finish_kernel after
+      // slice partials into the chunk totals; the end of this kernel (FINISH) or chunk_finish_kernel after
       // it adds them into Y
       tile_flush_partial(D, g, j0, kbe, acc, P.P + tl * dn);
     }
@@ -88,8 +88,9 @@ __global__ void __launch_bounds__(1024) tile_kernel(const TileGrid P, const __gr
   }
   // One-launch form for sketches too small for a second one: once every CTA's partials are in, the grid
   // finishes the chunk totals itself and writes all of Y. At 16384 x 16, d = 256, k = 4, FP32 the separate
-  // finish and the zeroing of Y took 7 of 20 us.
-  if (P.bar) {
+  // finish and the zeroing of Y took 7 of 20 us. An instantiation of its own, as this code costs the scatter
+  // loops of the other one 7 to 15 % (131072 x 65, d = 2080: 182 -> 201 us at k = 8, 79 -> 92 at k = 1).
+  if constexpr (FINISH) {
     if (!tile_grid_barrier(P.bar, P.status)) return;
     const int64_t nq = (D.n + 3) >> 2, quads = (int64_t)D.B * D.k * nq;
     for (int64_t f = (int64_t)threadIdx.x * gridDim.x + blockIdx.x; f < quads; f += (int64_t)gridDim.x * blockDim.x) {
@@ -102,6 +103,6 @@ __global__ void __launch_bounds__(1024) tile_kernel(const TileGrid P, const __gr
 using TileKernelFn = void (*)(const TileGrid, const CUtensorMap);
 
 // The tile kernel for a rule and a 16-bit element type of A (kAF16, kABF16), from sk_kernels_a16.cu.
-TileKernelFn tile_kernel_a16(int32_t rule, int32_t a_type);
+TileKernelFn tile_kernel_a16(int32_t rule, int32_t a_type, bool finish);
 
 }  // namespace sk
