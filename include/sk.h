@@ -106,7 +106,8 @@ typedef enum {
   SK_PARAM_DEVICE_STATUS = 9,
   /* Read-only: the kernel the last sketch ran: SK_KERNEL_TILE (1), SK_KERNEL_LITERAL (2),
    * SK_KERNEL_OWNER (3), SK_KERNEL_GLOBAL (4), 5 for the deterministic-mode kernel, or
-   * SK_KERNEL_REGISTER (6); 0 before the first sketch. */
+   * SK_KERNEL_REGISTER (6), 7 for the gather kernel (chunk accumulation by output rows, each row of A
+   * read by the owners of its target rows; AUTO only); 0 before the first sketch. */
   SK_PARAM_LAST_KERNEL = 10,
   /* Rows per group of sk_solve's tree QR (0, the default: as many rows as the GPU's shared memory
    * holds, so a sketch that fits is factored by one launch). Values below 2n are raised to 2n. */
@@ -115,7 +116,8 @@ typedef enum {
    * lambda + 1.5 sqrt(lambda) for lambda = box rows / B, the mean entries per row and box, e.g. 3 at
    * B = 512, where about 6 % of the entries overflow; 1..64 imposes it). Rows
    * beyond a full list are added into the chunk totals by FP32 vector reductions instead, with the
-   * same result up to FP32 summation order; small values exercise that path. */
+   * same result up to FP32 summation order; small values exercise that path.
+   * Gather kernel: list entries per owner (a half-warp, up to 8 output rows) and box. */
   SK_PARAM_LIST_CAP = 12,
   /* Upper bound, in bytes, on the device scratch this plan holds (0, the default: none). A call that
    * would grow the plan's scratch beyond it returns SK_ERR_OOM before enqueueing any work (Y is left

@@ -58,7 +58,7 @@ struct sk_plan_s {
   int64_t scratch_limit = 0;     // bound on the plan's device scratch in bytes (0: none)
   int64_t solve_wait_cycles = 0; // bound on each grid-barrier wait of the QR kernel (0: default)
   int64_t last_launches = 0, last_R = 0;
-  int32_t last_kernel = 0;  // kernel of the last sketch: 1 tile, 2 literal, 3 owner, 4 global, 5 deterministic
+  int32_t last_kernel = 0;  // kernel of the last sketch: 1 tile, 2 literal, 3 owner, 4 global, 5 deterministic, 6 register, 7 gather
   bool last_noalloc = false;  // the last sketch was an sk_apply_noalloc call (status in the static array)
   // device scratch
   float* det_P = nullptr;
@@ -141,7 +141,8 @@ struct TileCfg {
   bool own = false;
   bool vec = false;
   bool glob = false;
-  bool reg = false, reg_tile = false;
+  bool reg = false, gat = false;
+  bool other = false;  // chosen for speed: another kernel, which may need no chunk totals, runs where these cannot be had
   int32_t reg_nsub = 0, reg_cap = 0;
 };
 
@@ -189,15 +190,19 @@ int32_t choose_slices(const sk_plan_s* p, int64_t rows, int64_t R, int64_t ncg, 
 // fit in one round of CTAs, of at least 64 rows each. Below that size an item costs its CTA's start and its
 // flush of d x NC floats, and its rows hardly count; a 153rd item would cost a second round. Where one
 // slice needs no chunk totals (`finishes` false), only from three slices on, which pay for adding them up
-// (two were 2 us slower at 5000 x 256, d = 4096, k = 4). Measured, all slices at least 4096 rows / filled up
+// (two were 2 us slower at 5000 x 256, d = 4096, k = 4), and with n % 4 != 0, where every float of a flush is
+// an atomic of its own, only while an item's rows make as many additions (8192 x 130, d = 4160, k = 1, four
+// slices: 45 us, not 36). Measured, all slices at least 4096 rows / filled up
 // (and, but for the register kernel, one launch that finishes the chunk totals itself): 16384 x 16,
 // d = 256, k = 4 (4 items / 152): 42 / 14.5 us; 50001 x 33, d = 1056, k = 4 (16 / 144): 175 / 55;
 // 65536 x 64, d = 1024, k = 4 (32 / 144, register kernel): 47 / 28; 8192 x 64, d = 8192, k = 4: 43 / 28.
-int32_t fill_slices(const sk_plan_s* p, int64_t rows, int64_t R, int64_t ncg, int64_t nbg, int32_t cps,
+int32_t fill_slices(const sk_plan_s* p, int64_t n, int64_t rows, int64_t R, int64_t ncg, int64_t nbg, int32_t cps,
                     const DevInfo& di, int32_t slices, bool finishes) {
   const int64_t first = ((p->row_offset % R) + R) % R;
   const int64_t per = (first + rows + R - 1) / R * ncg * nbg;
-  const int64_t fit = std::min((int64_t)di.sms * std::max(cps, 1) / per, std::max<int64_t>(1, std::min(R, rows) / 64));
+  const int64_t chunk = std::min(R, rows);
+  int64_t fit = std::min((int64_t)di.sms * std::max(cps, 1) / per, std::max<int64_t>(1, chunk / 64));
+  if (n % 4 != 0) fit = std::min(fit, chunk * p->k / p->d);
   if (fit <= slices || (!finishes && slices == 1 && fit < 3)) return slices;
   return (int32_t)fit;
 }
@@ -251,7 +256,6 @@ void choose_global(const sk_plan_s* p, TileCfg* cfg) {
 // d = 4096 with k = 4 or 2 (B = 1024, 2048) the tile kernel stays ahead: 1416 vs 1357, 1735 vs 1448;
 // bfloat16 A: d = 4096, k = 8: 732 vs 1332 us; d = 1024, k = 4: 287 vs 735; 2^21 x 40, d = 320, k = 4:
 // 162 vs 356; 20000 x 128, d = 2048, k = 4: 26 vs 34; 2^18 x 1024, d = 2048, k = 4: 546 vs 917).
-// `reg_tile`: the tile kernel is the one to fall back to where chunk totals cannot be had (it may need none).
 bool choose_reg(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& di, bool tma_ok, int32_t a_type,
                 TileCfg* cfg) {
   if (p->mode != SK_MODE_ATOMIC || !tma_ok || rows >= ((int64_t)1 << 31)) return false;
@@ -273,17 +277,85 @@ bool choose_reg(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& di, 
   cfg->threads = reg_threads(a_type);
   cfg->R = R;
   cfg->long_slices = choose_slices(p, rows, R, ncg, ntg, 1, di);
-  cfg->slices = fill_slices(p, rows, R, ncg, ntg, 1, di, cfg->long_slices, true);
+  cfg->slices = fill_slices(p, n, rows, R, ncg, ntg, 1, di, cfg->long_slices, true);
   cfg->reg = true;
-  cfg->reg_tile = p->kernel == SK_KERNEL_AUTO && a_type != SK_A_FP32;
+  cfg->other = p->kernel == SK_KERNEL_AUTO && a_type != SK_A_FP32;
   cfg->reg_nsub = nsub;
   cfg->reg_cap = cap;
   return true;
 }
 
+// Where AUTO takes the gather kernel, by where it was the fastest (n from 4 to 1024, d / n = 2, 8, 32,
+// k = 1, 2, 4, 8, 2^13 to 2^22 rows; in brackets the time of the kernel taken otherwise over its time):
+// - aligned rows, n < 256, from 65536 rows on (8192 with d >= 4096, n >= 64: 1.3 to 1.4; below that its fixed
+//   cost loses up to 30 %): k = 1 from 24 columns on (1.1 to 3.2; 16 columns use a quarter of its lanes and
+//   need 2^20 rows: 1.2); k = 2 below the register kernel's 32 columns (1.0 to 1.35); k >= 2 where blocks are
+//   too tall for that kernel, B > 512 (k = 2 1.35 to 2.1; k = 4 1.2 to 1.4, while a row's k reads waste few
+//   lanes: 0.96 at n = 100); d from 8192 to 16383, FP32 (2^22 x 64, k = 8: 1.4);
+// - FP32, n >= 256, from 131072 rows on: k <= 2 with n <= 512 and d <= 2048 (1.03 to 1.6), k = 4 with B in
+//   (512, 1024] (2^19 x 1024: 1.27) or 2048 and n >= 512 (1.1), k = 8 with B in (512, 2048] (1.07 to 1.2);
+//   wider or taller the global kernel stays ahead;
+// - FP32 rows that TMA cannot read, from 32768 on: nearly everywhere (1.1 to 2.4; not with k = 8 and half of
+//   the last 64 columns empty, 0.88, nor with d above 8192 at k = 1); from 8192 on with k >= 2, n < 256 and d
+//   from 512 to 4224 (0.98 to 1.9).
+bool gather_wins(const sk_plan_s* p, int64_t n, int64_t rows, bool tma_ok, int32_t a_type) {
+  const int64_t k = p->k, d = p->d, B = p->B, lanes = (n + 63) / 64 * 64;
+  const bool f32 = a_type == SK_A_FP32;
+  if (rows >= ((int64_t)1 << 31) || rows < 8192 || B < 64 || k > 8 || n < 16) return false;
+  if (!tma_ok) {
+    if (!f32 || n < 17 || (k > 4 && 5 * n < 3 * lanes)) return false;
+    return rows >= 32768 ? k > 1 || d <= 8192 : k >= 2 && n < 256 && d >= 512 && d <= 4224;
+  }
+  if (n % 4 != 0 || (rows < 65536 && (d < 4096 || n < 64))) return false;
+  if (n < 256) {
+    if (k == 1) return (n >= 24 || rows >= (1 << 20)) && d <= 8192;
+    if (n < 32) return k == 2 && n >= 24;
+    if (B <= 512 || n < 48) return false;
+    return k * lanes <= 5 * n ? d <= 8192 : f32 && d >= 8192 && d < 16384;
+  }
+  if (!f32 || rows < 131072) return false;
+  if (k <= 2) return n <= 512 && d <= 2048;
+  if (B <= 512) return false;
+  return k <= 4 ? B <= (n >= 512 ? 2048 : 1024) : B <= 2048;
+}
+
+// Gather-kernel configuration. The slices are the ones for which the rounds of work items end first, an item
+// taking (measured at 2^22 x 64, d = 4096) 0.53 ns for each of its rows' hashes, 3.6 ns for each row it
+// fetches and 9 us to start and flush: k = 1, 2 / 7 / 14 slices 250 / 254 / 288 us, k = 4 611 / 544 / 565.
+bool choose_gather(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& di, bool tma_ok, int32_t a_type,
+                   TileCfg* cfg) {
+  if (p->mode != SK_MODE_ATOMIC || p->kernel != SK_KERNEL_AUTO || p->tile_cols != 0 || p->threads != 0 ||
+      !gather_wins(p, n, rows, tma_ok, a_type) ||
+      gat_smem_bytes(p->d, p->B, rows) > (size_t)std::min(di.optin, 232448) - 1024)
+    return false;
+  const int64_t R = p->R > 0 ? p->R : default_chunk_rows(p->m);
+  const int64_t ncg = (n + gat_cols() - 1) / gat_cols();
+  const int64_t tgs = gat_targets(p->d), ntg = (p->d + tgs - 1) / tgs;
+  const int64_t first = ((p->row_offset % R) + R) % R;
+  const int64_t chunks = (first + rows + R - 1) / R;
+  const double row_ns = 0.53 + 3.6 * (double)std::min<int64_t>(tgs, p->d) / (double)p->B;
+  const int64_t chunk = std::min(R, rows);
+  int64_t best = 1;
+  double best_ns = 1e300;
+  for (int64_t sl = 1; sl <= std::min<int64_t>(256, std::max<int64_t>(1, chunk / 64)); ++sl) {
+    const double rounds = (double)((chunks * sl * ncg * ntg + di.sms - 1) / di.sms);
+    const double ns = rounds * ((double)chunk / (double)sl * row_ns + 9000.0);
+    if (ns < best_ns) best_ns = ns, best = sl;
+  }
+  *cfg = TileCfg();
+  cfg->NC = 32;
+  cfg->kb = p->k;
+  cfg->R = R;
+  cfg->slices = cfg->long_slices = (int32_t)best;
+  cfg->reg_cap = p->list_cap;
+  cfg->gat = cfg->other = true;
+  return true;
+}
+
 sk_status choose_tile(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& di, TileCfg* cfg,
                       bool tma_ok = false, int32_t a_type = SK_A_FP32, bool scratch = true) {
-  if (choose_reg(p, n, rows, di, tma_ok, a_type, cfg) && (scratch || !cfg->reg_tile)) return SK_OK;
+  if (scratch && choose_gather(p, n, rows, di, tma_ok, a_type, cfg)) return SK_OK;
+  if (choose_reg(p, n, rows, di, tma_ok, a_type, cfg) && (scratch || !cfg->other)) return SK_OK;
   *cfg = TileCfg();
   if (p->kernel == SK_KERNEL_REGISTER)
     return set_error(SK_ERR_UNSUPPORTED,
@@ -322,7 +394,7 @@ sk_status choose_tile(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo
       cfg->grid = 0;
       cfg->R = R;
       cfg->long_slices = choose_slices(p, rows, R, 1, nbg, cps, di);
-      cfg->slices = fill_slices(p, rows, R, 1, nbg, cps, di, cfg->long_slices, false);
+      cfg->slices = fill_slices(p, n, rows, R, 1, nbg, cps, di, cfg->long_slices, false);
       cfg->depth = 1;
       cfg->mb = 1;
       cfg->serial = false;
@@ -400,7 +472,7 @@ sk_status choose_tile(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo
     const int64_t nbg = (p->k + kb - 1) / kb;
     const int32_t cps = tile_ctas_per_sm(p->rule, threads, tile_smem_bytes(p->B, kb, NC, threads, p->k, depth, mb));
     long_slices = choose_slices(p, rows, R, ncg, nbg, cps, di);
-    slices = fill_slices(p, rows, R, ncg, nbg, cps, di, long_slices, false);
+    slices = fill_slices(p, n, rows, R, ncg, nbg, cps, di, long_slices, false);
   }
   cfg->NC = NC;
   cfg->kb = kb;
@@ -526,7 +598,7 @@ sk_status enqueue_sketch(sk_plan_s* p, const void* A, int64_t lda, int64_t n, in
   const bool tma_ok = tma_layout_ok(A, lda, a_type == SK_A_FP32 ? 4 : 2);
   s = choose_tile(p, n, rows, di, &cfg, tma_ok, a_type);
   if (s != SK_OK) return s;
-  if (cfg.reg_tile && !totals_available(p, n, row_begin, row_end, R_fixed > 0 ? R_fixed : cfg.R, st)) {
+  if (cfg.other && !totals_available(p, n, row_begin, row_end, R_fixed > 0 ? R_fixed : cfg.R, st)) {
     s = choose_tile(p, n, rows, di, &cfg, tma_ok, a_type, false);
     if (s != SK_OK) return s;
   }
@@ -558,6 +630,7 @@ sk_status enqueue_sketch(sk_plan_s* p, const void* A, int64_t lda, int64_t n, in
   L.vec = cfg.vec ? 1 : 0;
   L.glob = cfg.glob ? 1 : 0;
   L.reg = cfg.reg ? 1 : 0;
+  L.gat = cfg.gat ? 1 : 0;
   L.reg_nsub = cfg.reg_nsub;
   L.reg_cap = cfg.reg_cap;
   L.col_off = col_off;
@@ -571,12 +644,12 @@ sk_status enqueue_sketch(sk_plan_s* p, const void* A, int64_t lda, int64_t n, in
   }
   L.status = p->dstatus;
   L.P = nullptr;
-  if (cfg.slices > 1 && cfg.long_slices == 1 && !cfg.glob && !cfg.reg) {
+  if (cfg.slices > 1 && cfg.long_slices == 1 && !cfg.glob && !cfg.reg && !cfg.gat) {
     // One launch, as with one slice per chunk, which needs no chunk totals and is taken where these cannot be had.
     if (totals_available(p, n, row_begin, row_end, cfg.R, st)) L.fuse_finish = zero_y ? 1 : 0;
     else L.slices = cfg.slices = 1;
   }
-  if (cfg.slices > 1 || cfg.glob || cfg.reg) {
+  if (cfg.slices > 1 || cfg.glob || cfg.reg || cfg.gat) {
     const size_t needP = sizeof(float) * (size_t)launch_P_floats(L);
     if (p->tileP_bytes < needP) {
       s = plan_grow(p, &p->tileP, &p->tileP_bytes, needP, "chunk-total scratch");
@@ -592,11 +665,12 @@ sk_status enqueue_sketch(sk_plan_s* p, const void* A, int64_t lda, int64_t n, in
   }
   cudaError_t e = launch_tile(L, st, launches);
   if (e != cudaSuccess)
-    return cuda_fail(e, cfg.glob  ? "global kernel launch"
+    return cuda_fail(e, cfg.gat   ? "gather kernel launch"
+                        : cfg.glob  ? "global kernel launch"
                         : cfg.reg ? "register kernel launch"
                         : cfg.own ? "owner kernel launch"
                                   : "tile kernel launch");
-  p->last_kernel = cfg.glob ? SK_KERNEL_GLOBAL : cfg.reg ? SK_KERNEL_REGISTER : cfg.own ? SK_KERNEL_OWNER : SK_KERNEL_TILE;
+  p->last_kernel = cfg.gat ? kGatherKernel : cfg.glob ? SK_KERNEL_GLOBAL : cfg.reg ? SK_KERNEL_REGISTER : cfg.own ? SK_KERNEL_OWNER : SK_KERNEL_TILE;
   if (R_used) *R_used = cfg.R;
   return SK_OK;
 }
@@ -1172,7 +1246,7 @@ sk_status sk_apply_partials(sk_plan p, const float* A, int64_t lda, int64_t n, f
     if (s != SK_OK) return s;
   }
   cfg.R = R;
-  if (!cfg.reg && cfg.slices < 2) cfg.slices = 2;  // work items flush into the chunk totals
+  if (!cfg.reg && !cfg.gat && cfg.slices < 2) cfg.slices = 2;  // work items flush into the chunk totals
   if (!p->dstatus) {
     size_t cur = 0;
     s = plan_grow(p, &p->dstatus, &cur, sizeof(unsigned), "status word");
@@ -1206,6 +1280,7 @@ sk_status sk_apply_partials(sk_plan p, const float* A, int64_t lda, int64_t n, f
   L.vec = cfg.vec ? 1 : 0;
   L.glob = 0;
   L.reg = cfg.reg ? 1 : 0;
+  L.gat = cfg.gat ? 1 : 0;
   L.reg_nsub = cfg.reg_nsub;
   L.reg_cap = cfg.reg_cap;
   L.col_off = 0;
@@ -1219,7 +1294,7 @@ sk_status sk_apply_partials(sk_plan p, const float* A, int64_t lda, int64_t n, f
   p->last_noalloc = false;
   p->last_launches = launches;
   p->last_R = R;
-  p->last_kernel = cfg.reg ? SK_KERNEL_REGISTER : cfg.own ? SK_KERNEL_OWNER : SK_KERNEL_TILE;
+  p->last_kernel = cfg.gat ? kGatherKernel : cfg.reg ? SK_KERNEL_REGISTER : cfg.own ? SK_KERNEL_OWNER : SK_KERNEL_TILE;
   return SK_OK;
 }
 
@@ -1316,8 +1391,13 @@ sk_status noalloc_tile_launch(const sk_plan_s* p, const float* A, int64_t lda, i
   s = dev_info(&di);
   if (s != SK_OK) return s;
   TileCfg cfg;
-  s = choose_tile(p, n, p->m, di, &cfg, tma_layout_ok(A, lda));  // FP32 A: never reg_tile
+  s = choose_tile(p, n, p->m, di, &cfg, tma_layout_ok(A, lda));
   if (s != SK_OK) return s;
+  const int64_t chunks = (p->row_offset + p->m - 1) / cfg.R - p->row_offset / cfg.R + 1;
+  if (cfg.other && sizeof(float) * (size_t)(chunks * p->d * n) > noalloc_P_bytes()) {
+    s = choose_tile(p, n, p->m, di, &cfg, tma_layout_ok(A, lda), SK_A_FP32, false);
+    if (s != SK_OK) return s;
+  }
   L->A = A;
   L->Y = Y;
   L->lda = lda;
@@ -1336,7 +1416,7 @@ sk_status noalloc_tile_launch(const sk_plan_s* p, const float* A, int64_t lda, i
   L->grid = cfg.grid;
   L->slices = cfg.slices;
   // One slice per chunk needs no chunk totals: taken where they would not fit in the static array.
-  if (cfg.slices > 1 && cfg.long_slices == 1 && !cfg.glob && !cfg.reg) {
+  if (cfg.slices > 1 && cfg.long_slices == 1 && !cfg.glob && !cfg.reg && !cfg.gat) {
     L->fuse_finish = 1;
     if (sizeof(float) * (size_t)launch_P_floats(*L) > noalloc_P_bytes()) L->fuse_finish = 0, L->slices = 1;
   }
@@ -1347,6 +1427,7 @@ sk_status noalloc_tile_launch(const sk_plan_s* p, const float* A, int64_t lda, i
   L->vec = cfg.vec ? 1 : 0;
   L->glob = cfg.glob ? 1 : 0;
   L->reg = cfg.reg ? 1 : 0;
+  L->gat = cfg.gat ? 1 : 0;
   L->reg_nsub = cfg.reg_nsub;
   L->reg_cap = cfg.reg_cap;
   L->col_off = 0;

@@ -196,7 +196,7 @@ int64_t launch_P_floats(const TileLaunch& L) {
     global_passes(L, &ns, &cb);
     return cb * L.d * ns;
   }
-  if (L.slices > 1 || L.reg) {
+  if (L.slices > 1 || L.reg || L.gat) {
     int64_t chunks;
     int32_t ncg, nbg;
     tile_geometry(L, &chunks, &ncg, &nbg);

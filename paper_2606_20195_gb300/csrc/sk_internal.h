@@ -8,6 +8,8 @@ namespace sk {
 
 struct TileDesc;
 
+constexpr int32_t kGatherKernel = 7;  // its number in SK_PARAM_LAST_KERNEL
+
 struct TileLaunch {
   const void* A;    // elements of type a_type (0 FP32, 1 binary16, 2 bfloat16)
   int32_t a_type = 0;
@@ -35,6 +37,7 @@ struct TileLaunch {
   int32_t glob = 0;   // 1: global-accumulator kernel (chunk totals in P, any d); needs P
   int32_t reg = 0;    // 1: register kernel (A through TMA; 32 columns x 1024 output rows per item, 16-bit A 64 x 512); needs P
   int32_t reg_nsub = 0, reg_cap = 0;  // register kernel: TMA copies per staged box, list entries per output row
+  int32_t gat = 0;    // 1: gather kernel (64 columns x up to 512 output rows per item); needs P
   int32_t fuse_finish = 0;  // 1: tile kernel with slices > 1 as one cooperative launch that also writes all of Y
   int32_t no_finish = 0;  // 1: leave the chunk totals in P (no chunk-finish launch); P is then the caller's
 };
@@ -78,6 +81,12 @@ int32_t reg_cols(int32_t a_type);
 bool reg_choose_box(int64_t d, int64_t B, int32_t a_type, size_t smem_limit, int32_t cap_fixed, int32_t* nsub,
                     int32_t* cap);
 cudaError_t launch_reg(const TileLaunch& L, cudaStream_t st, int32_t* launches);
+// Gather kernel (sk_gather.cu): output rows and columns per work item, shared-memory bytes for items of
+// `rows` rows, and the launch (its chunk finish included; needs L.P; L.reg_cap > 0 imposes the list capacity).
+int32_t gat_targets(int64_t d);
+int32_t gat_cols();
+size_t gat_smem_bytes(int64_t d, int64_t B, int64_t rows);
+cudaError_t launch_gather(const TileLaunch& L, cudaStream_t st, int32_t* launches);
 // Resident CTAs per SM of the tile kernel for (rule, threads, dynamic shared memory).
 int32_t tile_ctas_per_sm(int32_t rule, int32_t threads, size_t smem);
 
