@@ -86,11 +86,16 @@ typedef enum {
    * SK_KERNEL_REGISTER (chunk accumulation in registers: every thread owns one output row x 32
    * columns of a 1024-row group, rows of A are routed to their owners through per-row lists in shared
    * memory, no floating-point atomics on chip; needs FP32 A, 16-byte aligned with lda a multiple of 4, and
-   * atomic mode; SK_ERR_UNSUPPORTED otherwise). AUTO takes the register kernel for FP32 A with
+   * atomic mode; SK_ERR_UNSUPPORTED otherwise). AUTO takes the register kernel (for a
+   * 16-bit A its form with 512 output rows and 64 columns per work item) for
    * k >= 2, n >= 32 and B = d/k <= 512 (except n >= 256 with k = 2) when A's layout allows TMA
-   * (and neither SK_PARAM_TILE_COLS nor SK_PARAM_THREADS is set); otherwise the tile kernel, or the global kernel when a block of S is
-   * too tall for the tile kernel's shared-memory accumulator, when the tile kernel would need several
-   * block groups or only 4-column items of a matrix with n >= 256, and for n >= 256 at k <= 2. */
+   * (and neither SK_PARAM_TILE_COLS nor SK_PARAM_THREADS is set); the gather kernel (every output row has
+   * one owner, which reads the rows of A that S sends to it; AUTO only) for most other sketches of at
+   * least 65536 rows, and of FP32 rows that TMA cannot read from 8192 to 32768 rows on; otherwise the
+   * tile kernel, or the global kernel when a block of S is too tall for the tile kernel's shared-memory
+   * accumulator, when the tile kernel would need several block groups or only 4-column items of a matrix
+   * with n >= 256, and for n >= 256 at k <= 2. The register kernel for 16-bit A and the gather kernel need
+   * chunk-total scratch; where the scratch limit or a stream capture leaves none, another kernel runs. */
   SK_PARAM_KERNEL = 4,
   /* Columns per work item of the tile kernel (4, 8, 16 or 32; 0 = automatic). */
   SK_PARAM_TILE_COLS = 5,

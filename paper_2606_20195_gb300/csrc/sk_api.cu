@@ -322,6 +322,10 @@ bool gather_wins(const sk_plan_s* p, int64_t n, int64_t rows, bool tma_ok, int32
 // Gather-kernel configuration. The slices are the ones for which the rounds of work items end first, an item
 // taking (measured at 2^22 x 64, d = 4096) 0.53 ns for each of its rows' hashes, 3.6 ns for each row it
 // fetches and 9 us to start and flush: k = 1, 2 / 7 / 14 slices 250 / 254 / 288 us, k = 4 611 / 544 / 565.
+// Few slices make long FP32 sums: of an output's N = chunk / B additions a slice makes N / s one after another,
+// and the chunk total s. The squared error grows with N / s + s, least at s = sqrt(N); slices that make it more
+// than 3 % larger than that are not taken (2^21 x 128, d = 4096, k = 4: tile kernel with 19 slices 1.25e-7,
+// here with 25 % allowed 1.34e-7).
 bool choose_gather(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& di, bool tma_ok, int32_t a_type,
                    TileCfg* cfg) {
   if (p->mode != SK_MODE_ATOMIC || p->kernel != SK_KERNEL_AUTO || p->tile_cols != 0 || p->threads != 0 ||
@@ -335,9 +339,12 @@ bool choose_gather(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& d
   const int64_t chunks = (first + rows + R - 1) / R;
   const double row_ns = 0.53 + 3.6 * (double)std::min<int64_t>(tgs, p->d) / (double)p->B;
   const int64_t chunk = std::min(R, rows);
-  int64_t best = 1;
+  const double adds = (double)chunk / (double)p->B, adds_max = std::max(4.0, 2.06 * std::sqrt(adds));
+  const int64_t most = std::min<int64_t>(1024, std::max<int64_t>(1, chunk / 64));
+  int64_t best = std::min(most, std::max<int64_t>(1, (int64_t)std::sqrt(adds)));
   double best_ns = 1e300;
-  for (int64_t sl = 1; sl <= std::min<int64_t>(256, std::max<int64_t>(1, chunk / 64)); ++sl) {
+  for (int64_t sl = 1; sl <= std::min<int64_t>(most, 256); ++sl) {
+    if (adds / (double)sl + (double)sl > adds_max) continue;
     const double rounds = (double)((chunks * sl * ncg * ntg + di.sms - 1) / di.sms);
     const double ns = rounds * ((double)chunk / (double)sl * row_ns + 9000.0);
     if (ns < best_ns) best_ns = ns, best = sl;
