@@ -290,11 +290,11 @@ bool choose_reg(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& di, 
 // - aligned rows, n < 256, from 65536 rows on (8192 with d >= 4096, n >= 64: 1.3 to 1.4; below that its fixed
 //   cost loses up to 30 %): k = 1 from 24 columns on (1.1 to 3.2; 16 columns use a quarter of its lanes and
 //   need 2^20 rows: 1.2); k = 2 below the register kernel's 32 columns (1.0 to 1.35); k >= 2 where blocks are
-//   too tall for that kernel, B > 512 (k = 2 1.35 to 2.1; k = 4 1.2 to 1.4, while a row's k reads waste few
+//   too tall for that kernel, B > 512 (k = 2 1.25 to 1.8; k = 4 1.1 to 1.3, while a row's k reads waste few
 //   lanes: 0.96 at n = 100); d from 8192 to 16383, FP32 (2^22 x 64, k = 8: 1.4);
-// - FP32, n >= 256, from 131072 rows on: k <= 2 with n <= 512 and d <= 2048 (1.03 to 1.6), k = 4 with B in
-//   (512, 1024] (2^19 x 1024: 1.27) or 2048 and n >= 512 (1.1), k = 8 with B in (512, 2048] (1.07 to 1.2);
-//   wider or taller the global kernel stays ahead;
+// - FP32, n >= 256, from 131072 rows on: k <= 2 with n <= 512 and d <= 2048 (d <= 2 n 1.02 to 1.6; d above
+//   that from 2^20 rows on 1.13 to 1.3, at 131072 rows 0.85), k = 3 or 4 with B in (512, 1024] (2^19 x 1024:
+//   1.12); elsewhere the global kernel stays ahead (k = 8, d = 16384: 0.83);
 // - FP32 rows that TMA cannot read, from 32768 on: nearly everywhere (1.1 to 2.4; not with k = 8 and half of
 //   the last 64 columns empty, 0.88, nor with d above 8192 at k = 1); from 8192 on with k >= 2, n < 256 and d
 //   from 512 to 4224 (0.98 to 1.9).
@@ -314,9 +314,8 @@ bool gather_wins(const sk_plan_s* p, int64_t n, int64_t rows, bool tma_ok, int32
     return k * lanes <= 5 * n ? d <= 8192 : f32 && d >= 8192 && d < 16384;
   }
   if (!f32 || rows < 131072) return false;
-  if (k <= 2) return n <= 512 && d <= 2048;
-  if (B <= 512) return false;
-  return k <= 4 ? B <= (n >= 512 ? 2048 : 1024) : B <= 2048;
+  if (k <= 2) return n <= 512 && d <= 2048 && (d <= 2 * n || rows >= (1 << 20));
+  return k <= 4 && B > 512 && B <= 1024;
 }
 
 // Gather-kernel configuration. The slices are the ones for which the rounds of work items end first, an item

@@ -25,10 +25,10 @@
 // box before they fetch and half after, so that hashing and memory latency overlap.
 // What bounds it: at k = 1 the loads in flight (64 KB a CTA; 4.1 TB/s at 2^22 x 64), at k = 4 the L1 data path
 // (k |A| through it) and the sums' shared-memory traffic. Boxes of about 64 entries per half-warp: with 32 the
-// barrier waits for the longest list (k = 4: 616 us against 544), with 96 the lists take the shared memory that
+// barrier waits for the longest list (k = 4, 7 slices: 616 us against 544), with 96 the lists take the shared memory that
 // the L1 cache needs for rows in flight (614 us).
-// Measured at 2^22 x 64, d = 4096 (before: tile kernel): k = 1 516 -> 263 us, k = 2 618 -> 350, k = 4 759 -> 565;
-// 2^19 x 1024, d = 4096, k = 4 1659 -> 1304; 50001 x 33 (unaligned rows), d = 1056, k = 4 55 -> 39 us (175 before short slices).
+// Measured at 2^22 x 64, d = 4096 (before: tile kernel): k = 1 516 -> 264 us, k = 2 618 -> 369, k = 4 759 -> 582;
+// 2^19 x 1024, d = 4096, k = 4 1659 -> 1487; 50001 x 33 (unaligned rows), d = 1056, k = 4 55 -> 39 us (175 before short slices).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
