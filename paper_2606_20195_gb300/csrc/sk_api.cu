@@ -68,6 +68,10 @@ struct sk_plan_s {
   double* lsqr = nullptr;       // sk_solve_precond: u (m), 8 n-vectors, scalars, x0 (n floats)
   size_t lsqr_bytes = 0;
   size_t tileP_bytes = 0;
+  // one-launch sketches: the words of the grid barrier, then chunk totals (all zero between launches). The words
+  // stay at one place whatever n and d: totals may end as -0, which is zero as a number and not as a counter.
+  unsigned* fastP = nullptr;
+  size_t fastP_bytes = 0;
   void* solve_buf = nullptr;
   size_t solve_bytes = 0;
   size_t solve_status_off = 0, solve_kappa_off = 0;
@@ -108,7 +112,7 @@ size_t elem_size(int32_t rule) { return rule == SK_FP32 ? 4 : 2; }
 
 // Device scratch the plan holds, in bytes.
 size_t plan_scratch_bytes(const sk_plan_s* p) {
-  return p->det_P_bytes + (p->dstatus ? sizeof(unsigned) : 0) + p->tileP_bytes + p->lsqr_bytes + p->solve_bytes +
+  return p->det_P_bytes + (p->dstatus ? sizeof(unsigned) : 0) + p->tileP_bytes + p->fastP_bytes + p->lsqr_bytes + p->solve_bytes +
          2 * p->stage_bytes + p->ydev_bytes;
 }
 
@@ -515,9 +519,17 @@ sk_status validate_apply(const sk_plan_s* p, const void* A, int64_t lda, int64_t
 // scratch limit, and not while the stream is being captured.
 bool totals_available(const sk_plan_s* p, int64_t n, int64_t row_begin, int64_t row_end, int64_t R, cudaStream_t st) {
   const int64_t chunks = (row_end - 1) / R - row_begin / R + 1;
-  const size_t need = sizeof(float) * (size_t)(chunks * p->d * n + kBarrierFloats);
+  const size_t need = sizeof(float) * (size_t)(chunks * p->d * n);
   if (p->tileP_bytes >= need) return true;
   if (p->scratch_limit > 0 && plan_scratch_bytes(p) - p->tileP_bytes + need > (size_t)p->scratch_limit) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+}
+
+// The same for the barrier words and totals of a one-launch sketch.
+bool fast_totals_available(const sk_plan_s* p, size_t need, cudaStream_t st) {
+  if (p->fastP_bytes >= need) return true;
+  if (p->scratch_limit > 0 && plan_scratch_bytes(p) - p->fastP_bytes + need > (size_t)p->scratch_limit) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   return cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
 }
@@ -651,11 +663,22 @@ sk_status enqueue_sketch(sk_plan_s* p, const void* A, int64_t lda, int64_t n, in
   L.status = p->dstatus;
   L.P = nullptr;
   if (cfg.slices > 1 && cfg.long_slices == 1 && !cfg.glob && !cfg.reg && !cfg.gat) {
-    // One launch, as with one slice per chunk, which needs no chunk totals and is taken where these cannot be had.
-    if (totals_available(p, n, row_begin, row_end, cfg.R, st)) L.fuse_finish = zero_y ? 1 : 0;
-    else L.slices = cfg.slices = 1;
-  }
-  if (cfg.slices > 1 || cfg.glob || cfg.reg || cfg.gat) {
+    // One slice per chunk needs no chunk totals and is taken where these cannot be had. The short slices finish
+    // in the same launch if Y is this call's alone (not with a Y that other calls add to as well).
+    const size_t need = sizeof(float) * (size_t)(kBarrierWords + launch_P_floats(L));
+    if (fast_totals_available(p, need, st)) {
+      if (p->fastP_bytes < need) {
+        s = plan_grow(p, &p->fastP, &p->fastP_bytes, need, "chunk-total scratch");
+        if (s != SK_OK) return s;
+        cudaError_t ez = cudaMemsetAsync(p->fastP, 0, need, st);
+        if (ez != cudaSuccess) return cuda_fail(ez, "zeroing chunk totals");
+      }
+      L.P = reinterpret_cast<float*>(p->fastP) + kBarrierWords;
+      if (zero_y) L.bar = p->fastP;
+    } else {
+      L.slices = cfg.slices = 1;
+    }
+  } else if (cfg.slices > 1 || cfg.glob || cfg.reg || cfg.gat) {
     const size_t needP = sizeof(float) * (size_t)launch_P_floats(L);
     if (p->tileP_bytes < needP) {
       s = plan_grow(p, &p->tileP, &p->tileP_bytes, needP, "chunk-total scratch");
@@ -665,7 +688,7 @@ sk_status enqueue_sketch(sk_plan_s* p, const void* A, int64_t lda, int64_t n, in
     }
     L.P = p->tileP;
   }
-  if (zero_y && !L.fuse_finish) {
+  if (zero_y && !L.bar) {
     cudaError_t ez = cudaMemsetAsync(Y, 0, elem_size(p->rule) * (size_t)(p->d * n), st);
     if (ez != cudaSuccess) return cuda_fail(ez, "zeroing Y");
   }
@@ -1370,6 +1393,7 @@ void sk_destroy(sk_plan p) {
   if (p->det_P) cudaFree(p->det_P);
   if (p->dstatus) cudaFree(p->dstatus);
   if (p->tileP) cudaFree(p->tileP);
+  if (p->fastP) cudaFree(p->fastP);
   if (p->lsqr) cudaFree(p->lsqr);
   if (p->solve_buf) cudaFree(p->solve_buf);
   for (int b = 0; b < 2; ++b) {
@@ -1388,7 +1412,10 @@ namespace sk {
 
 // Tile-kernel launch description for sk_apply_noalloc (sk_noalloc.cu): the same configuration
 // sk_apply's atomic tile path chooses, with no scratch attached. Allocates nothing.
-sk_status noalloc_tile_launch(const sk_plan_s* p, const float* A, int64_t lda, int64_t n, void* Y, TileLaunch* L) {
+// `one_launch`: the caller is to attach the words of a grid barrier (TileLaunch::bar) behind the totals.
+sk_status noalloc_tile_launch(const sk_plan_s* p, const float* A, int64_t lda, int64_t n, void* Y, TileLaunch* L,
+                              bool* one_launch) {
+  *one_launch = false;
   sk_status s = validate_apply(p, A, lda, n, Y);
   if (s != SK_OK) return s;
   if (p->mode != SK_MODE_ATOMIC || p->kernel == SK_KERNEL_LITERAL)
@@ -1423,8 +1450,8 @@ sk_status noalloc_tile_launch(const sk_plan_s* p, const float* A, int64_t lda, i
   L->slices = cfg.slices;
   // One slice per chunk needs no chunk totals: taken where they would not fit in the static array.
   if (cfg.slices > 1 && cfg.long_slices == 1 && !cfg.glob && !cfg.reg && !cfg.gat) {
-    L->fuse_finish = 1;
-    if (sizeof(float) * (size_t)launch_P_floats(*L) > noalloc_P_bytes()) L->fuse_finish = 0, L->slices = 1;
+    *one_launch = sizeof(float) * (size_t)(launch_P_floats(*L) + kBarrierWords) <= noalloc_P_bytes();
+    if (!*one_launch) L->slices = 1;
   }
   L->depth = cfg.depth;
   L->mb = cfg.mb;

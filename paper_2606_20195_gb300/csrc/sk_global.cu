@@ -200,7 +200,7 @@ int64_t launch_P_floats(const TileLaunch& L) {
     int64_t chunks;
     int32_t ncg, nbg;
     tile_geometry(L, &chunks, &ncg, &nbg);
-    return chunks * L.d * L.n + (L.fuse_finish ? kBarrierFloats : 0);
+    return chunks * L.d * L.n;
   }
   return 0;
 }

@@ -38,7 +38,8 @@ struct TileLaunch {
   int32_t reg = 0;    // 1: register kernel (A through TMA; 32 columns x 1024 output rows per item, 16-bit A 64 x 512); needs P
   int32_t reg_nsub = 0, reg_cap = 0;  // register kernel: TMA copies per staged box, list entries per output row
   int32_t gat = 0;    // 1: gather kernel (64 columns x up to 512 output rows per item); needs P
-  int32_t fuse_finish = 0;  // 1: tile kernel with slices > 1 as one cooperative launch that also writes all of Y
+  unsigned* bar = nullptr;  // tile kernel with slices > 1: kBarrierWords zero words; one cooperative launch then
+                            // finishes the chunk totals too and writes all of Y
   int32_t no_finish = 0;  // 1: leave the chunk totals in P (no chunk-finish launch); P is then the caller's
 };
 
@@ -67,8 +68,8 @@ void tile_geometry(const TileLaunch& L, int64_t* chunks, int32_t* ncg, int32_t* 
 // Passes of the global-accumulator kernel: column slabs of *ns columns and batches of *cb chunks,
 // chosen so that the chunk totals of one pass (cb x d x ns FP32) stay resident in L2.
 void global_passes(const TileLaunch& L, int64_t* ns, int64_t* cb);
-constexpr int64_t kBarrierFloats = 2;
-// FP32 elements of chunk-total scratch P a launch needs (0: none), with the barrier words of fuse_finish.
+constexpr int64_t kBarrierWords = 64;  // 2 in use; 256 bytes keep what follows aligned
+// FP32 elements of chunk-total scratch P a launch needs (0: none).
 int64_t launch_P_floats(const TileLaunch& L);
 // The global-accumulator kernel and its chunk finish, in passes (sk_global.cu); needs L.P.
 cudaError_t launch_global(const TileLaunch& L, cudaStream_t st, int32_t* launches);

@@ -116,7 +116,7 @@ cudaError_t launch_tile(const TileLaunch& L, cudaStream_t st, int32_t* launches)
   P.acc_floats = (int32_t)tile_acc_floats((uint32_t)B, L.kb, P.D.S, L.NC);
   P.P = L.P;
   P.chunks = chunks;
-  P.bar = nullptr;
+  P.bar = L.bar;
   P.status = L.status;
   P.D.col_off = L.col_off;
   P.D.a_type = L.a_type;
@@ -143,7 +143,7 @@ cudaError_t launch_tile(const TileLaunch& L, cudaStream_t st, int32_t* launches)
   int sms = 0;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  const bool finish = L.fuse_finish && P.slices > 1;
+  const bool finish = L.bar != nullptr && P.slices > 1;
   const TileKernelFn kern = L.a_type != kAF32 ? tile_kernel_a16(L.rule, L.a_type, finish)
                             : finish            ? tile_kernel_f32<true>(L.rule)
                                                 : tile_kernel_f32<false>(L.rule);
@@ -158,7 +158,6 @@ cudaError_t launch_tile(const TileLaunch& L, cudaStream_t st, int32_t* launches)
   grid = std::min<int64_t>(grid, P.items);
   if (grid < 1) grid = 1;
   if (finish) {
-    P.bar = reinterpret_cast<unsigned*>(L.P + chunks * L.d * L.n);
     void* args[2] = {&P, &tmap};
     e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(kern), dim3((unsigned)grid), dim3(L.threads), args,
                                     smem, st);

@@ -8,7 +8,8 @@
 #include "sk_internal.h"
 
 namespace sk {
-sk_status noalloc_tile_launch(const sk_plan_s* p, const float* A, int64_t lda, int64_t n, void* Y, TileLaunch* L);
+sk_status noalloc_tile_launch(const sk_plan_s* p, const float* A, int64_t lda, int64_t n, void* Y, TileLaunch* L,
+                              bool* one_launch);
 size_t noalloc_elem_size(const sk_plan_s* p);
 void noalloc_record(sk_plan_s* p, int64_t launches, int64_t R, int32_t kernel);
 sk_status noalloc_read_status(unsigned* out);
@@ -42,12 +43,13 @@ extern "C" SK_API sk_status sk_apply_noalloc(sk_plan p, const float* A, int64_t 
                                              void* stream) {
   clear_error();
   TileLaunch L;
-  sk_status s = noalloc_tile_launch(p, A, lda, n, Y, &L);
+  bool one_launch = false;
+  sk_status s = noalloc_tile_launch(p, A, lda, n, Y, &L, &one_launch);
   if (s != SK_OK) return s;
   void* base = nullptr;
   s = scratch_address(&base);
   if (s != SK_OK) return s;
-  const size_t need_P = sizeof(float) * (size_t)launch_P_floats(L);
+  const size_t need_P = sizeof(float) * (size_t)(launch_P_floats(L) + (one_launch ? kBarrierWords : 0));
   if (need_P > noalloc_P_bytes())
     return set_error(SK_ERR_UNSUPPORTED,
                      "sk_apply_noalloc: this size needs %zu bytes of scratch, above the %zu-byte static array; "
@@ -62,6 +64,7 @@ extern "C" SK_API sk_status sk_apply_noalloc(sk_plan p, const float* A, int64_t 
   if (e != cudaSuccess) return set_error(SK_ERR_CUDA, "zeroing: %s", cudaGetErrorString(e));
   L.status = reinterpret_cast<unsigned*>(b);
   L.P = need_P ? reinterpret_cast<float*>(b + kStatusBytes) : nullptr;
+  if (one_launch) L.bar = reinterpret_cast<unsigned*>(L.P + launch_P_floats(L));
   int32_t launches = 0;
   e = launch_tile(L, st, &launches);
   if (e != cudaSuccess) return set_error(SK_ERR_CUDA, "sketch kernel launch: %s", cudaGetErrorString(e));

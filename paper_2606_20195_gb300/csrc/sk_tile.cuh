@@ -63,7 +63,7 @@ struct TileGrid {
   int32_t use_tma;             // 1: A arrives through the tensor map
   int32_t depth;               // TMA ring slots per warp
   int64_t chunks;              // chunks of the launch
-  unsigned* bar;               // cooperative launch: two zero counters of the grid barrier; null: no finish here
+  unsigned* bar;               // one-launch finish: kBarrierWords zero words of its grid barrier
 };
 
 // Per-warp TMA staging ring: `depth` slots of RB x NC floats (128-byte aligned) and their mbarriers.

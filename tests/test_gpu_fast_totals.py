@@ -1,0 +1,63 @@
+"""Sketches that AUTO finishes in one launch (short slices of each chunk; past a grid barrier the same kernel adds
+the chunk totals into Y): the launch count and the scratch show that this form ran, and one plan serves matrices of
+different width and height in turn, growing and shrinking, with data whose chunk totals cancel to subnormal
+numbers of either sign in between (an FP32 reduction leaves -0 there). Integer data, so every chunk total is
+exact and the result is bit-exact with the oracle's canonical order."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+BARRIER = 256  # bytes of barrier words in front of the chunk totals
+
+
+def _bits(Y, rule):
+    import torch
+    return Y.cpu().numpy() if rule == 0 else Y.view(torch.int16).cpu().numpy().view(np.uint16)
+
+
+def _ints(m, n, seed):
+    return np.random.default_rng(seed).integers(-3, 4, size=(m, n)).astype(np.float32)
+
+
+@pytest.mark.parametrize("shape", [(16384, 16, 256, 4), (5001, 33, 48, 4), (9000, 20, 64, 1), (4097, 1, 256, 4),
+                                   (8000, 64, 8192, 4), (3000, 12, 4096, 2), (200, 5, 16, 1)])
+@pytest.mark.parametrize("rule", [0, 2])
+def test_one_launch(sk, dev, shape, rule):
+    import torch
+    m, n, d, k = shape
+    A = _ints(m, n, m + n)
+    plan = sk.Plan(d, m, k, rule, 11)
+    Y = torch.full((d, n), 7.0, dtype=plan.out_dtype(), device=dev)
+    for _ in range(2):  # the second call finds barrier words and totals cleared
+        plan.apply(torch.from_numpy(A).to(dev), Y)
+    torch.cuda.synchronize()
+    R = plan.get(sk.SK_PARAM_LAST_CHUNK_ROWS)
+    assert plan.get(sk.SK_PARAM_LAST_LAUNCHES) == 1 and plan.get(sk.SK_PARAM_LAST_KERNEL) == sk.SK_KERNEL_TILE
+    assert plan.get(sk.SK_PARAM_SCRATCH_BYTES) == 4 + BARRIER + 4 * -(-m // R) * d * n
+    assert plan.get(sk.SK_PARAM_DEVICE_STATUS) == 0
+    assert np.array_equal(_bits(Y, rule), oracle.sketch_canonical(A, d, k, 11, rule, R))
+    plan.close()
+
+
+def test_one_plan_many_widths(sk, dev):
+    import torch
+    d, k, rule = 256, 4, 0
+    plan = sk.Plan(d, 16384, k, rule, 11)
+    rng = np.random.default_rng(2)
+    for i, (m, n) in enumerate([(16384, 16), (9000, 12), (16384, 16), (4096, 20), (16384, 24), (5000, 4), (12000, 20)]):
+        plan.set(sk.SK_PARAM_ROWS, m)
+        # neighbouring rows cancel to a few units of 2^-136: totals that end as subnormals or signed zeros
+        tiny = np.repeat(1.0 + rng.integers(0, 8, (m // 2, n)) * 2.0 ** -10, 2, axis=0) * 2.0 ** -126
+        tiny[1::2] *= -1.0
+        tiny = np.ascontiguousarray(tiny + (rng.integers(0, 3, tiny.shape) - 1) * 2.0 ** -136).astype(np.float32)
+        Y = torch.empty((d, n), device=dev)
+        plan.apply(torch.from_numpy(tiny).to(dev), Y)
+        A = _ints(m, n, i)
+        plan.apply(torch.from_numpy(A).to(dev), Y)
+        torch.cuda.synchronize()
+        assert plan.get(sk.SK_PARAM_LAST_LAUNCHES) == 1
+        assert np.array_equal(Y.cpu().numpy(), oracle.sketch_canonical(A, d, k, 11, rule, plan.get(sk.SK_PARAM_LAST_CHUNK_ROWS)))
+    assert plan.get(sk.SK_PARAM_DEVICE_STATUS) == 0
+    plan.close()
