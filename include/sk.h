@@ -128,9 +128,11 @@ typedef enum {
    * would grow the plan's scratch beyond it returns SK_ERR_OOM before enqueueing any work (Y is left
    * as it was); for services that admit work under a device-memory budget. */
   SK_PARAM_SCRATCH_LIMIT = 13,
-  /* Upper bound, in SM clock cycles, on each grid-barrier wait of sk_solve's QR kernel (0, the
-   * default: about two seconds). A barrier that gives up ends the kernel and sk_solve_status returns
-   * SK_ERR_TIMEOUT; small values exist to exercise that path. */
+  /* Upper bound, in SM clock cycles, on each grid-barrier wait of sk_solve's QR kernel and of small
+   * sketches that finish in one launch (0, the default: about two seconds). A barrier that gives up ends
+   * the kernel and sk_solve_status returns SK_ERR_TIMEOUT (a sketch sets bit 0 of
+   * SK_PARAM_DEVICE_STATUS, its Y is invalid, and the next call is unaffected); small values exist to
+   * exercise that path. */
   SK_PARAM_SOLVE_WAIT_CYCLES = 14,
   /* Read-only: bytes of device scratch the plan holds now. */
   SK_PARAM_SCRATCH_BYTES = 15,

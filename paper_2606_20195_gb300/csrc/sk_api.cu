@@ -56,7 +56,7 @@ struct sk_plan_s {
   int64_t solve_group_rows = 0;  // rows per QR group of sk_solve (0: as many as shared memory holds)
   int32_t list_cap = 0;          // register kernel: list entries per output row and box (0: automatic)
   int64_t scratch_limit = 0;     // bound on the plan's device scratch in bytes (0: none)
-  int64_t solve_wait_cycles = 0; // bound on each grid-barrier wait of the QR kernel (0: default)
+  int64_t solve_wait_cycles = 0; // bound on each grid-barrier wait (0: default)
   int64_t last_launches = 0, last_R = 0;
   int32_t last_kernel = 0;  // kernel of the last sketch: 1 tile, 2 literal, 3 owner, 4 global, 5 deterministic, 6 register, 7 gather
   bool last_noalloc = false;  // the last sketch was an sk_apply_noalloc call (status in the static array)
@@ -675,6 +675,7 @@ sk_status enqueue_sketch(sk_plan_s* p, const void* A, int64_t lda, int64_t n, in
       }
       L.P = reinterpret_cast<float*>(p->fastP) + kBarrierWords;
       if (zero_y) L.bar = p->fastP;
+      L.wait_cycles = p->solve_wait_cycles;
     } else {
       L.slices = cfg.slices = 1;
     }

@@ -40,6 +40,7 @@ struct TileLaunch {
   int32_t gat = 0;    // 1: gather kernel (64 columns x up to 512 output rows per item); needs P
   unsigned* bar = nullptr;  // tile kernel with slices > 1: kBarrierWords zero words; one cooperative launch then
                             // finishes the chunk totals too and writes all of Y
+  int64_t wait_cycles = 0;  // bound on the grid-barrier wait of that launch (0: default)
   int32_t no_finish = 0;  // 1: leave the chunk totals in P (no chunk-finish launch); P is then the caller's
 };
 

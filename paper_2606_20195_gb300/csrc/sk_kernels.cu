@@ -117,6 +117,7 @@ cudaError_t launch_tile(const TileLaunch& L, cudaStream_t st, int32_t* launches)
   P.P = L.P;
   P.chunks = chunks;
   P.bar = L.bar;
+  P.wait_cycles = L.wait_cycles > 0 ? L.wait_cycles : 4ll << 30;  // about two seconds
   P.status = L.status;
   P.D.col_off = L.col_off;
   P.D.a_type = L.a_type;

@@ -64,6 +64,7 @@ struct TileGrid {
   int32_t depth;               // TMA ring slots per warp
   int64_t chunks;              // chunks of the launch
   unsigned* bar;               // one-launch finish: kBarrierWords zero words of its grid barrier
+  long long wait_cycles;       // bound on the wait of that barrier
 };
 
 // Per-warp TMA staging ring: `depth` slots of RB x NC floats (128-byte aligned) and their mbarriers.

@@ -8,18 +8,22 @@ namespace sk {
 
 // ------------------------------------------------------------------ tile kernel
 
-// Wait until every CTA of a co-resident (cooperative) grid has arrived; bar[0] counts arrivals, bar[1]
-// departures, and the last CTA to depart clears both for the next launch. Writes before the call are
-// visible to every CTA after it. Gives up after about two seconds (then false, and the status word says so).
-__device__ __forceinline__ bool tile_grid_barrier(unsigned* bar, unsigned* status) {
-  __shared__ int ok;
+// Wait until every CTA of a co-resident (cooperative) grid has arrived. Writes before the call are visible to
+// every CTA after it. bar[0] counts arrivals, bar[1] departures and, from bit 16 on, those of CTAs that gave up,
+// after `limit` SM clock cycles (false is returned then, and the status word says so). The last CTA to depart,
+// when all have arrived and added what they had to add, clears both words and, if one gave up, the `totals`
+// floats at `P` too: whatever happened, the next launch finds them at zero. (A grid has fewer than 2^16 CTAs,
+// being resident at once. A word of its own for those that gave up cost the last CTA a microsecond.)
+__device__ __forceinline__ bool tile_grid_barrier(unsigned* bar, unsigned* status, long long limit, float* P,
+                                                  int64_t totals) {
+  __shared__ int ok, clean;
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
     ok = 0;
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
     const long long t0 = clock64();
-    while (clock64() - t0 < (4ll << 30)) {
+    while (clock64() - t0 < limit) {
       unsigned v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
       if (v >= gridDim.x) {
@@ -28,12 +32,19 @@ __device__ __forceinline__ bool tile_grid_barrier(unsigned* bar, unsigned* statu
       }
     }
     if (!ok && status) atomicOr(status, kStatusTimeout);
-    if (ok && atomicAdd(bar + 1, 1u) == gridDim.x - 1) {
+    clean = 0;
+    const unsigned left = atomicAdd(bar + 1, ok ? 1u : 0x10001u);
+    if ((left & 0xFFFFu) == gridDim.x - 1) {
       bar[0] = 0u;
       bar[1] = 0u;
+      clean = !ok || (left >> 16) != 0u;
     }
   }
   __syncthreads();
+  if (clean) {
+    __threadfence();
+    for (int64_t i = threadIdx.x; i < totals; i += blockDim.x) __stcg(P + i, 0.f);
+  }
   return ok != 0;
 }
 
@@ -91,7 +102,7 @@ __global__ void __launch_bounds__(1024) tile_kernel(const TileGrid P, const __gr
   // finish and the zeroing of Y took 7 of 20 us. An instantiation of its own, as this code costs the scatter
   // loops of the other one 7 to 15 % (131072 x 65, d = 2080: 182 -> 201 us at k = 8, 79 -> 92 at k = 1).
   if constexpr (FINISH) {
-    if (!tile_grid_barrier(P.bar, P.status)) return;
+    if (!tile_grid_barrier(P.bar, P.status, P.wait_cycles, P.P, P.chunks * dn)) return;
     const int64_t nq = (D.n + 3) >> 2, quads = (int64_t)D.B * D.k * nq;
     for (int64_t f = (int64_t)threadIdx.x * gridDim.x + blockIdx.x; f < quads; f += (int64_t)gridDim.x * blockDim.x) {
       const int64_t r = f / nq;

@@ -61,3 +61,23 @@ def test_one_plan_many_widths(sk, dev):
         assert np.array_equal(Y.cpu().numpy(), oracle.sketch_canonical(A, d, k, 11, rule, plan.get(sk.SK_PARAM_LAST_CHUNK_ROWS)))
     assert plan.get(sk.SK_PARAM_DEVICE_STATUS) == 0
     plan.close()
+
+
+@pytest.mark.parametrize("shape", [(16384, 16, 256, 4), (5001, 33, 48, 4), (4097, 1, 256, 4)])
+def test_call_after_a_barrier_gave_up(sk, dev, shape):
+    # A barrier wait of one cycle runs out; the next call on the plan must find its scratch clean.
+    import torch
+    m, n, d, k = shape
+    A = _ints(m, n, 3)
+    plan = sk.Plan(d, m, k, 1, 11, solve_wait_cycles=1)
+    Ad, Y = torch.from_numpy(A).to(dev), torch.empty((d, n), dtype=torch.float16, device=dev)
+    for _ in range(3):
+        plan.apply(Ad, Y)
+    assert plan.get(sk.SK_PARAM_DEVICE_STATUS) == 1
+    plan.set(sk.SK_PARAM_SOLVE_WAIT_CYCLES, 0)
+    for _ in range(2):
+        plan.apply(Ad, Y)
+        torch.cuda.synchronize()
+        assert plan.get(sk.SK_PARAM_LAST_LAUNCHES) == 1
+        assert np.array_equal(_bits(Y, 1), oracle.sketch_canonical(A, d, k, 11, 1, plan.get(sk.SK_PARAM_LAST_CHUNK_ROWS)))
+    plan.close()
