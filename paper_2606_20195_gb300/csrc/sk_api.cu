@@ -68,8 +68,9 @@ struct sk_plan_s {
   double* lsqr = nullptr;       // sk_solve_precond: u (m), 8 n-vectors, scalars, x0 (n floats)
   size_t lsqr_bytes = 0;
   size_t tileP_bytes = 0;
-  // one-launch sketches: the words of the grid barrier, then chunk totals (all zero between launches). The words
-  // stay at one place whatever n and d: totals may end as -0, which is zero as a number and not as a counter.
+  // for sketches that could do without chunk totals: the words of the one-launch form's grid barrier, then the
+  // totals (all zero between launches). The words stay at one place whatever n and d: totals may end as -0,
+  // which is zero as a number and not as a counter.
   unsigned* fastP = nullptr;
   size_t fastP_bytes = 0;
   void* solve_buf = nullptr;
@@ -148,6 +149,7 @@ struct TileCfg {
   bool reg = false, gat = false;
   bool other = false;  // chosen for speed: another kernel, which may need no chunk totals, runs where these cannot be had
   int32_t reg_nsub = 0, reg_cap = 0;
+  bool tile_alone() const { return !glob && !reg && !gat && !own; }
 };
 
 // Default chunk length: at most 8 chunks per matrix (each output then receives at most 8 rounded
@@ -515,23 +517,39 @@ sk_status validate_apply(const sk_plan_s* p, const void* A, int64_t lda, int64_t
   return SK_OK;
 }
 
-// Whether the chunk totals of a sketch with chunk length R are in place or may be allocated: within the
-// scratch limit, and not while the stream is being captured.
-bool totals_available(const sk_plan_s* p, int64_t n, int64_t row_begin, int64_t row_end, int64_t R, cudaStream_t st) {
-  const int64_t chunks = (row_end - 1) / R - row_begin / R + 1;
-  const size_t need = sizeof(float) * (size_t)(chunks * p->d * n);
-  if (p->tileP_bytes >= need) return true;
-  if (p->scratch_limit > 0 && plan_scratch_bytes(p) - p->tileP_bytes + need > (size_t)p->scratch_limit) return false;
+bool capturing(cudaStream_t st) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
 }
 
-// The same for the barrier words and totals of a one-launch sketch.
-bool fast_totals_available(const sk_plan_s* p, size_t need, cudaStream_t st) {
-  if (p->fastP_bytes >= need) return true;
-  if (p->scratch_limit > 0 && plan_scratch_bytes(p) - p->fastP_bytes + need > (size_t)p->scratch_limit) return false;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+// Chunk-total bytes of a sketch with chunk length R.
+size_t totals_bytes(const sk_plan_s* p, int64_t n, int64_t row_begin, int64_t row_end, int64_t R) {
+  return sizeof(float) * (size_t)(((row_end - 1) / R - row_begin / R + 1) * p->d * n);
+}
+
+// Whether a buffer of the plan (`cur` bytes now) holds `need` bytes or may be grown to: within the scratch
+// limit, and not while the stream is being captured.
+bool can_hold(const sk_plan_s* p, size_t cur, size_t need, cudaStream_t st) {
+  if (cur >= need) return true;
+  if (p->scratch_limit > 0 && plan_scratch_bytes(p) - cur + need > (size_t)p->scratch_limit) return false;
+  return !capturing(st);
+}
+
+// *P = the `need` bytes of chunk totals in p->fastP, for a sketch that can do without any; null where they are
+// not to be had. Not in a stream capture, even with the buffer in place: the graph would hold its address,
+// which a later call that needs a larger one frees.
+sk_status take_fast(sk_plan_s* p, size_t need, cudaStream_t st, float** P) {
+  *P = nullptr;
+  need += sizeof(unsigned) * kBarrierWords;
+  if (capturing(st) || !can_hold(p, p->fastP_bytes, need, st)) return SK_OK;
+  if (p->fastP_bytes < need) {
+    sk_status s = plan_grow(p, &p->fastP, &p->fastP_bytes, need, "chunk-total scratch");
+    if (s != SK_OK) return s;
+    cudaError_t ez = cudaMemsetAsync(p->fastP, 0, need, st);
+    if (ez != cudaSuccess) return cuda_fail(ez, "zeroing chunk totals");
+  }
+  *P = reinterpret_cast<float*>(p->fastP + kBarrierWords);
+  return SK_OK;
 }
 
 // Enqueue Y = S * A for rows [row_begin, row_begin + rows) (A row 0 = row_begin) with chunk rows R.
@@ -616,12 +634,38 @@ sk_status enqueue_sketch(sk_plan_s* p, const void* A, int64_t lda, int64_t n, in
   const bool tma_ok = tma_layout_ok(A, lda, a_type == SK_A_FP32 ? 4 : 2);
   s = choose_tile(p, n, rows, di, &cfg, tma_ok, a_type);
   if (s != SK_OK) return s;
-  if (cfg.other && !totals_available(p, n, row_begin, row_end, R_fixed > 0 ? R_fixed : cfg.R, st)) {
-    s = choose_tile(p, n, rows, di, &cfg, tma_ok, a_type, false);
-    if (s != SK_OK) return s;
-  }
   if (cfg.own && a_type != SK_A_FP32) return set_error(SK_ERR_UNSUPPORTED, "the owner kernel reads FP32 A only");
   if (R_fixed > 0) cfg.R = R_fixed;
+  if (!p->dstatus) {
+    size_t cur = 0;
+    s = plan_grow(p, &p->dstatus, &cur, sizeof(unsigned), "status word");
+    if (s != SK_OK) return s;
+    cudaError_t ez = cudaMemsetAsync(p->dstatus, 0, sizeof(unsigned), st);
+    if (ez != cudaSuccess) return cuda_fail(ez, "zeroing status word");
+  }
+  // Chunk totals of a sketch that another kernel, or one slice per chunk, makes without any: taken if they can
+  // be had, else that form runs. (Sketches that need totals either way keep them in p->tileP.)
+  float* fast = nullptr;
+  if (cfg.other) {
+    TileCfg alt;
+    s = choose_tile(p, n, rows, di, &alt, tma_ok, a_type, false);
+    if (s != SK_OK) return s;
+    if (R_fixed > 0) alt.R = R_fixed;
+    bool ok;
+    if (alt.tile_alone() && alt.long_slices == 1) {
+      alt.slices = 1;
+      s = take_fast(p, totals_bytes(p, n, row_begin, row_end, cfg.R), st, &fast);
+      if (s != SK_OK) return s;
+      ok = fast != nullptr;
+    } else {
+      ok = can_hold(p, p->tileP_bytes, totals_bytes(p, n, row_begin, row_end, cfg.R), st);
+    }
+    if (!ok) cfg = alt;
+  } else if (cfg.tile_alone() && cfg.slices > 1 && cfg.long_slices == 1) {
+    s = take_fast(p, totals_bytes(p, n, row_begin, row_end, cfg.R), st, &fast);
+    if (s != SK_OK) return s;
+    if (!fast) cfg.slices = 1;
+  }
   TileLaunch L;
   L.A = A;
   L.a_type = a_type;
@@ -653,32 +697,12 @@ sk_status enqueue_sketch(sk_plan_s* p, const void* A, int64_t lda, int64_t n, in
   L.reg_cap = cfg.reg_cap;
   L.col_off = col_off;
   L.allow_tma = cfg.vec ? 0 : 1;
-  if (!p->dstatus) {
-    size_t cur = 0;
-    s = plan_grow(p, &p->dstatus, &cur, sizeof(unsigned), "status word");
-    if (s != SK_OK) return s;
-    cudaError_t ez = cudaMemsetAsync(p->dstatus, 0, sizeof(unsigned), st);
-    if (ez != cudaSuccess) return cuda_fail(ez, "zeroing status word");
-  }
   L.status = p->dstatus;
-  L.P = nullptr;
-  if (cfg.slices > 1 && cfg.long_slices == 1 && !cfg.glob && !cfg.reg && !cfg.gat) {
-    // One slice per chunk needs no chunk totals and is taken where these cannot be had. The short slices finish
-    // in the same launch if Y is this call's alone (not with a Y that other calls add to as well).
-    const size_t need = sizeof(float) * (size_t)(kBarrierWords + launch_P_floats(L));
-    if (fast_totals_available(p, need, st)) {
-      if (p->fastP_bytes < need) {
-        s = plan_grow(p, &p->fastP, &p->fastP_bytes, need, "chunk-total scratch");
-        if (s != SK_OK) return s;
-        cudaError_t ez = cudaMemsetAsync(p->fastP, 0, need, st);
-        if (ez != cudaSuccess) return cuda_fail(ez, "zeroing chunk totals");
-      }
-      L.P = reinterpret_cast<float*>(p->fastP) + kBarrierWords;
-      if (zero_y) L.bar = p->fastP;
-      L.wait_cycles = p->solve_wait_cycles;
-    } else {
-      L.slices = cfg.slices = 1;
-    }
+  L.P = fast;
+  if (fast) {
+    // The short slices finish in the same launch if Y is this call's alone (not one that other calls add to).
+    if (zero_y && cfg.tile_alone()) L.bar = p->fastP;
+    L.wait_cycles = p->solve_wait_cycles;
   } else if (cfg.slices > 1 || cfg.glob || cfg.reg || cfg.gat) {
     const size_t needP = sizeof(float) * (size_t)launch_P_floats(L);
     if (p->tileP_bytes < needP) {

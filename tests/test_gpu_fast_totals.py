@@ -81,3 +81,32 @@ def test_call_after_a_barrier_gave_up(sk, dev, shape):
         assert plan.get(sk.SK_PARAM_LAST_LAUNCHES) == 1
         assert np.array_equal(_bits(Y, 1), oracle.sketch_canonical(A, d, k, 11, 1, plan.get(sk.SK_PARAM_LAST_CHUNK_ROWS)))
     plan.close()
+
+
+@pytest.mark.parametrize("shape", [(16384, 16, 256, 4), (33000, 33, 1056, 4)])
+def test_graph_outlives_the_plans_scratch(sk, dev, shape):
+    # A graph captured after an eager call replays after a larger call has made the plan's scratch grow.
+    import torch
+    m, n, d, k = shape
+    A, B = _ints(m, n, 1), _ints(m, 4 * n, 2)
+    Ad, Bd = torch.from_numpy(A).to(dev), torch.from_numpy(B).to(dev)
+    plan = sk.Plan(d, m, k, 1, 11)
+    Y = torch.empty((d, n), dtype=torch.float16, device=dev)
+    Z = torch.empty((d, 4 * n), dtype=torch.float16, device=dev)
+    plan.apply(Ad, Y)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        plan.apply(Ad, Y)
+    plan.apply(Bd, Z)
+    torch.cuda.synchronize()
+    for _ in range(2):
+        Y.zero_()
+        graph.replay()
+        plan.apply(Bd, Z)
+        torch.cuda.synchronize()
+        R = plan.get(sk.SK_PARAM_LAST_CHUNK_ROWS)
+        assert np.array_equal(_bits(Y, 1), oracle.sketch_canonical(A, d, k, 11, 1, R))
+        assert np.array_equal(_bits(Z, 1), oracle.sketch_canonical(B, d, k, 11, 1, R))
+    assert plan.get(sk.SK_PARAM_DEVICE_STATUS) == 0
+    plan.close()

@@ -1,0 +1,77 @@
+"""Which kernel a sketch takes and what scratch it touches, on the host side alone: libsk runs over a CUDA runtime
+without a GPU (tests/fake_cudart.c, preloaded in a child process) that counts launches and allocations and can be
+told that a stream is being captured, that earlier work is still running, or that an allocation fails. Kernels are
+not run, so nothing here says anything about results."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+PRELUDE = """
+import ctypes, sys
+sys.path.insert(0, %r)
+from paper_2606_20195_gb300 import sk
+fake = ctypes.CDLL(None)
+def var(name, t=ctypes.c_int): return t.in_dll(fake, name)
+capturing, busy, most = var("fake_capturing"), var("fake_busy"), var("fake_max", ctypes.c_ulonglong)
+kernels, coop, mallocs, frees = var("fake_kernels"), var("fake_coop"), var("fake_mallocs"), var("fake_frees")
+GATHER, BAR = 7, 256
+A, Y, ST = 1 << 20, 1 << 21, 64  # addresses that nothing reads
+SMALL = dict(d=256, m=16384, k=4), 16      # one launch (short slices), else one slice per chunk
+GATH = dict(d=4096, m=65536, k=1), 128     # gather kernel, else the tile kernel with one slice per chunk
+REG16 = dict(d=512, m=4000, k=4), 64       # register kernel for a 16-bit A, else the tile kernel
+BOTH = dict(d=4096, m=1 << 22, k=1), 64    # gather kernel, else the tile kernel with chunk totals too
+def totals(case, chunks): return 4 * chunks * case[0]["d"] * case[1]
+def apply(p, n, st=ST, a_type=0, lda=None):
+    c0, k0 = coop.value, kernels.value
+    if a_type: sk.sk_apply_typed(p.handle, A, a_type, lda or n, n, Y, st)
+    else: sk.sk_apply(p.handle, A, lda or n, n, Y, st)
+    return p.get(sk.SK_PARAM_LAST_KERNEL), coop.value - c0, kernels.value - k0
+def plan(case, rule=1, **kw): return sk.Plan(case[0]["d"], case[0]["m"], case[0]["k"], rule, 1, **kw)
+def held(p): return p.get(sk.SK_PARAM_SCRATCH_BYTES)
+TILE, REG, GLOBAL = sk.SK_KERNEL_TILE, sk.SK_KERNEL_REGISTER, sk.SK_KERNEL_GLOBAL
+""" % ROOT
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    from paper_2606_20195_gb300 import _build
+    _build.build()
+    lib = str(tmp_path_factory.mktemp("fake") / "fake_cudart.so")
+    subprocess.run(["gcc", "-O1", "-shared", "-fPIC", "-Wno-builtin-declaration-mismatch", "-o", lib,
+                    os.path.join(HERE, "fake_cudart.c")], check=True)
+
+    def go(body):
+        r = subprocess.run([sys.executable, "-c", PRELUDE + body], capture_output=True, text=True,
+                           env={**os.environ, "LD_PRELOAD": lib, "CUDA_VISIBLE_DEVICES": ""})
+        assert r.returncode == 0, r.stdout + r.stderr
+    return go
+
+
+def test_routes(run):
+    run("""
+p = plan(SMALL); assert apply(p, 16) == (TILE, 1, 0) and held(p) == 4 + BAR + totals(SMALL, 4), held(p)
+p = plan(GATH); assert apply(p, 128)[0] == GATHER and held(p) == 4 + BAR + totals(GATH, 8), held(p)
+p = plan(REG16); assert apply(p, 64, a_type=1)[0] == REG and held(p) == 4 + BAR + totals(REG16, 1), held(p)
+p = plan(BOTH); assert apply(p, 64)[0] == GATHER and held(p) == 4 + totals(BOTH, 8), held(p)
+""")
+
+
+def test_capture_takes_no_scratch_that_a_later_call_may_free(run):
+    # A graph keeps the addresses of its launches. Sketches that need no chunk totals must not put totals into
+    # one, even where the plan has them already: a later, larger call frees the buffer.
+    run("""
+for case, n, t in ((SMALL, 16, 0), (GATH, 128, 0), (REG16, 64, 1)):
+    p = plan(case); first = apply(p, n, a_type=t); before = held(p)
+    capturing.value = 1
+    assert apply(p, n, a_type=t) == (TILE, 0, 1)
+    assert held(p) == before
+    capturing.value = 0
+    assert apply(p, n, a_type=t) == first
+p = plan(BOTH); first = apply(p, 64); capturing.value = 1
+assert apply(p, 64) == first  # (needs the plan's totals in either form)
+""")
