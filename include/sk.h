@@ -23,6 +23,9 @@
  *     sk_last_error() then holds a message for the calling thread. Asynchronous device faults
  *     surface as SK_ERR_CUDA on a later call. Nothing aborts the process.
  *   - A plan may be used from one host thread at a time; distinct plans are independent.
+ *     Calls of one plan on several streams share its scratch (chunk totals, solve workspace): order
+ *     them, unless they are sketches that need no chunk totals (the tile kernel with one slice per
+ *     chunk), which take optional totals only while no other stream's call of the plan may use them.
  */
 #ifndef SK_H_
 #define SK_H_

@@ -73,6 +73,8 @@ struct sk_plan_s {
   // which is zero as a number and not as a counter.
   unsigned* fastP = nullptr;
   size_t fastP_bytes = 0;
+  cudaEvent_t fast_done = nullptr;     // behind the last call that used fastP,
+  unsigned long long fast_stream = 0;  // and the id of its stream (ids, unlike handles, are not used again)
   void* solve_buf = nullptr;
   size_t solve_bytes = 0;
   size_t solve_status_off = 0, solve_kappa_off = 0;
@@ -535,13 +537,33 @@ bool can_hold(const sk_plan_s* p, size_t cur, size_t need, cudaStream_t st) {
   return !capturing(st);
 }
 
+// For the calls inside its scope, another stream's capture in global mode is no error (this thread's stream is
+// not the captured one): the allocations and queries made for optional scratch must not end it.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // *P = the `need` bytes of chunk totals in p->fastP, for a sketch that can do without any; null where they are
 // not to be had. Not in a stream capture, even with the buffer in place: the graph would hold its address,
-// which a later call that needs a larger one frees.
+// which a later call that needs a larger one frees. And not while a call on another stream may still be using
+// them: without totals a sketch touches only its own A and Y, so one thread may issue several with one plan on
+// several streams. The caller launches on st next and then calls leave_fast.
 sk_status take_fast(sk_plan_s* p, size_t need, cudaStream_t st, float** P) {
   *P = nullptr;
   need += sizeof(unsigned) * kBarrierWords;
   if (capturing(st) || !can_hold(p, p->fastP_bytes, need, st)) return SK_OK;
+  unsigned long long id = 0;
+  if (cudaStreamGetId(st, &id) != cudaSuccess) return cudaGetLastError(), SK_OK;
+  RelaxedCapture relaxed;
+  if (!p->fast_done) {
+    if (cudaEventCreateWithFlags(&p->fast_done, cudaEventDisableTiming) != cudaSuccess) return cudaGetLastError(), SK_OK;
+  } else if (id != p->fast_stream && cudaEventQuery(p->fast_done) != cudaSuccess) {
+    cudaGetLastError();
+    return SK_OK;
+  }
+  p->fast_stream = id;
   if (p->fastP_bytes < need) {
     sk_status s = plan_grow(p, &p->fastP, &p->fastP_bytes, need, "chunk-total scratch");
     if (s != SK_OK) return s;
@@ -550,6 +572,12 @@ sk_status take_fast(sk_plan_s* p, size_t need, cudaStream_t st, float** P) {
   }
   *P = reinterpret_cast<float*>(p->fastP + kBarrierWords);
   return SK_OK;
+}
+
+// The call's launches on st that use p->fastP are enqueued.
+sk_status leave_fast(sk_plan_s* p, cudaStream_t st) {
+  cudaError_t e = cudaEventRecord(p->fast_done, st);
+  return e == cudaSuccess ? SK_OK : cuda_fail(e, "chunk-total scratch");
 }
 
 // Enqueue Y = S * A for rows [row_begin, row_begin + rows) (A row 0 = row_begin) with chunk rows R.
@@ -718,6 +746,10 @@ sk_status enqueue_sketch(sk_plan_s* p, const void* A, int64_t lda, int64_t n, in
     if (ez != cudaSuccess) return cuda_fail(ez, "zeroing Y");
   }
   cudaError_t e = launch_tile(L, st, launches);
+  if (fast) {
+    s = leave_fast(p, st);
+    if (e == cudaSuccess && s != SK_OK) return s;
+  }
   if (e != cudaSuccess)
     return cuda_fail(e, cfg.gat   ? "gather kernel launch"
                         : cfg.glob  ? "global kernel launch"
@@ -1419,6 +1451,7 @@ void sk_destroy(sk_plan p) {
   if (p->dstatus) cudaFree(p->dstatus);
   if (p->tileP) cudaFree(p->tileP);
   if (p->fastP) cudaFree(p->fastP);
+  if (p->fast_done) cudaEventDestroy(p->fast_done);
   if (p->lsqr) cudaFree(p->lsqr);
   if (p->solve_buf) cudaFree(p->solve_buf);
   for (int b = 0; b < 2; ++b) {

@@ -110,3 +110,59 @@ def test_graph_outlives_the_plans_scratch(sk, dev, shape):
         assert np.array_equal(_bits(Z, 1), oracle.sketch_canonical(B, d, k, 11, 1, R))
     assert plan.get(sk.SK_PARAM_DEVICE_STATUS) == 0
     plan.close()
+
+
+@pytest.mark.parametrize("shape", [(16384, 16, 256, 4), (33000, 33, 1056, 4), (8000, 64, 8192, 4)])
+def test_one_plan_on_several_streams(sk, dev, shape):
+    # Nothing orders the streams' calls, and each has its own A and Y. (Sketches that need no chunk totals; those of
+    # the register kernel for FP32 A, say, always share the plan's.)
+    import torch
+    m, n, d, k = shape
+    plan = sk.Plan(d, m, k, 1, 11)
+    streams = [torch.cuda.Stream() for _ in range(4)]
+    A = [_ints(m, n, s) for s in range(4)]
+    Ad = [torch.from_numpy(a).to(dev) for a in A]
+    Y = [[torch.empty((d, n), dtype=torch.float16, device=dev) for _ in range(8)] for _ in range(4)]
+    plan.apply(Ad[0], Y[0][0])
+    torch.cuda.synchronize()
+    for i in range(8):
+        for s in range(4):
+            plan.apply(Ad[s], Y[s][i], streams[s])
+    torch.cuda.synchronize()
+    assert plan.get(sk.SK_PARAM_DEVICE_STATUS) == 0
+    R = plan.get(sk.SK_PARAM_LAST_CHUNK_ROWS)
+    for s in range(4):
+        ref = oracle.sketch_canonical(A[s], d, k, 11, 1, R)
+        for i in range(8):
+            assert np.array_equal(_bits(Y[s][i], 1), ref), (s, i)
+    plan.close()
+
+
+def test_eager_call_beside_another_streams_capture(sk, dev):
+    # The scratch of an eager call is allocated while another stream is being captured (global mode).
+    import torch
+    m, n, d, k = 16384, 16, 256, 4
+    A = _ints(m, n, 1)
+    Ad = torch.from_numpy(A).to(dev)
+    first, plan = sk.Plan(d, m, k, 1, 11), sk.Plan(d, m, k, 1, 11)
+    Y, Z = (torch.zeros((d, n), dtype=torch.float16, device=dev) for _ in range(2))
+    side = torch.cuda.Stream()
+    first.apply(Ad, Z)
+    small = torch.from_numpy(A[:64]).to(dev)
+    plan.set(sk.SK_PARAM_ROWS, 64)
+    plan.apply(small, Y)  # (the plan's status word)
+    plan.set(sk.SK_PARAM_ROWS, m)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        first.apply(Ad, Z)
+        plan.apply(Ad, Y, side)
+    torch.cuda.synchronize()
+    ref = oracle.sketch_canonical(A, d, k, 11, 1, plan.get(sk.SK_PARAM_LAST_CHUNK_ROWS))
+    assert np.array_equal(_bits(Y, 1), ref)
+    Z.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(_bits(Z, 1), ref)
+    first.close()
+    plan.close()

@@ -75,3 +75,16 @@ for case, n, t in ((SMALL, 16, 0), (GATH, 128, 0), (REG16, 64, 1)):
 p = plan(BOTH); first = apply(p, 64); capturing.value = 1
 assert apply(p, 64) == first  # (needs the plan's totals in either form)
 """)
+
+
+def test_another_streams_totals_are_left_alone(run):
+    run("""
+for case, n, t in ((SMALL, 16, 0), (GATH, 128, 0), (REG16, 64, 1)):
+    p = plan(case); fast = apply(p, n, 64, t); busy.value = 1
+    assert apply(p, n, 64, t) == fast            # the same stream: in order
+    assert apply(p, n, 128, t) == (TILE, 0, 1)   # another one, while the first may be running
+    assert apply(p, n, 64, t) == fast
+    busy.value = 0
+    assert apply(p, n, 128, t) == fast; busy.value = 1
+    assert apply(p, n, 64, t) == (TILE, 0, 1); busy.value = 0
+""")
