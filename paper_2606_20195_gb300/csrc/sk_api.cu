@@ -545,33 +545,34 @@ struct RelaxedCapture {
   ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
 };
 
-// *P = the `need` bytes of chunk totals in p->fastP, for a sketch that can do without any; null where they are
-// not to be had. Not in a stream capture, even with the buffer in place: the graph would hold its address,
+// A buffer of chunk totals of the plan with room for `need` bytes, zero where it is new. False where the memory
+// is not to be had: no error yet, as the caller may have a form that needs less.
+template <typename T>
+bool grow_totals(sk_plan_s* p, T** ptr, size_t* cur, size_t need, cudaStream_t st) {
+  if (*cur >= need) return true;
+  if (plan_grow(p, ptr, cur, need, "chunk-total scratch") != SK_OK) return clear_error(), false;
+  return cudaMemsetAsync(*ptr, 0, need, st) == cudaSuccess;
+}
+
+// The `need` bytes of chunk totals in p->fastP, for a sketch that can do without any; null where they are not to
+// be had. Not in a stream capture, even with the buffer in place: the graph would hold its address,
 // which a later call that needs a larger one frees. And not while a call on another stream may still be using
 // them: without totals a sketch touches only its own A and Y, so one thread may issue several with one plan on
 // several streams. The caller launches on st next and then calls leave_fast.
-sk_status take_fast(sk_plan_s* p, size_t need, cudaStream_t st, float** P) {
-  *P = nullptr;
+float* take_fast(sk_plan_s* p, size_t need, cudaStream_t st) {
   need += sizeof(unsigned) * kBarrierWords;
-  if (capturing(st) || !can_hold(p, p->fastP_bytes, need, st)) return SK_OK;
+  if (capturing(st) || !can_hold(p, p->fastP_bytes, need, st)) return nullptr;
   unsigned long long id = 0;
-  if (cudaStreamGetId(st, &id) != cudaSuccess) return cudaGetLastError(), SK_OK;
+  if (cudaStreamGetId(st, &id) != cudaSuccess) return cudaGetLastError(), nullptr;
   RelaxedCapture relaxed;
   if (!p->fast_done) {
-    if (cudaEventCreateWithFlags(&p->fast_done, cudaEventDisableTiming) != cudaSuccess) return cudaGetLastError(), SK_OK;
+    if (cudaEventCreateWithFlags(&p->fast_done, cudaEventDisableTiming) != cudaSuccess) return cudaGetLastError(), nullptr;
   } else if (id != p->fast_stream && cudaEventQuery(p->fast_done) != cudaSuccess) {
-    cudaGetLastError();
-    return SK_OK;
+    return cudaGetLastError(), nullptr;
   }
   p->fast_stream = id;
-  if (p->fastP_bytes < need) {
-    sk_status s = plan_grow(p, &p->fastP, &p->fastP_bytes, need, "chunk-total scratch");
-    if (s != SK_OK) return s;
-    cudaError_t ez = cudaMemsetAsync(p->fastP, 0, need, st);
-    if (ez != cudaSuccess) return cuda_fail(ez, "zeroing chunk totals");
-  }
-  *P = reinterpret_cast<float*>(p->fastP + kBarrierWords);
-  return SK_OK;
+  if (!grow_totals(p, &p->fastP, &p->fastP_bytes, need, st)) return nullptr;
+  return reinterpret_cast<float*>(p->fastP + kBarrierWords);
 }
 
 // The call's launches on st that use p->fastP are enqueued.
@@ -682,16 +683,15 @@ sk_status enqueue_sketch(sk_plan_s* p, const void* A, int64_t lda, int64_t n, in
     bool ok;
     if (alt.tile_alone() && alt.long_slices == 1) {
       alt.slices = 1;
-      s = take_fast(p, totals_bytes(p, n, row_begin, row_end, cfg.R), st, &fast);
-      if (s != SK_OK) return s;
+      fast = take_fast(p, totals_bytes(p, n, row_begin, row_end, cfg.R), st);
       ok = fast != nullptr;
     } else {
-      ok = can_hold(p, p->tileP_bytes, totals_bytes(p, n, row_begin, row_end, cfg.R), st);
+      const size_t need = totals_bytes(p, n, row_begin, row_end, cfg.R);
+      ok = can_hold(p, p->tileP_bytes, need, st) && grow_totals(p, &p->tileP, &p->tileP_bytes, need, st);
     }
     if (!ok) cfg = alt;
   } else if (cfg.tile_alone() && cfg.slices > 1 && cfg.long_slices == 1) {
-    s = take_fast(p, totals_bytes(p, n, row_begin, row_end, cfg.R), st, &fast);
-    if (s != SK_OK) return s;
+    fast = take_fast(p, totals_bytes(p, n, row_begin, row_end, cfg.R), st);
     if (!fast) cfg.slices = 1;
   }
   TileLaunch L;

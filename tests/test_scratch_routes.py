@@ -88,3 +88,16 @@ for case, n, t in ((SMALL, 16, 0), (GATH, 128, 0), (REG16, 64, 1)):
     assert apply(p, n, 128, t) == fast; busy.value = 1
     assert apply(p, n, 64, t) == (TILE, 0, 1); busy.value = 0
 """)
+
+
+def test_a_failed_allocation_takes_the_form_that_needs_less(run):
+    run("""
+most.value = 1 << 15  # cudaMalloc of more than this fails
+for case, n, t in ((SMALL, 16, 0), (GATH, 128, 0), (REG16, 64, 1)):
+    p = plan(case)
+    assert apply(p, n, a_type=t) == (TILE, 0, 1) and held(p) == 4
+WIDE = dict(d=8192, m=65536, k=2), 257  # gather kernel, else the global kernel, in passes with smaller totals
+p = plan(WIDE); most.value = 0; assert apply(p, 257)[0] == GATHER; need = held(p) - 4
+p = plan(WIDE); most.value = need - 1
+assert apply(p, 257)[0] == GLOBAL and 4 < held(p) < 4 + need
+""")
