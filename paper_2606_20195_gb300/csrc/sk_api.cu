@@ -215,6 +215,19 @@ int32_t fill_slices(const sk_plan_s* p, int64_t n, int64_t rows, int64_t R, int6
   return (int32_t)fit;
 }
 
+// Whether the chunks of `rows` rows are long enough for a kernel whose chunk totals another form would do
+// without: the default chunk length always (at most 8 chunks, one more with a row offset, of at least 4096
+// rows); shorter ones the caller has set while the totals are no larger than A in FP32, and many of them while
+// a quarter of it. So what a plan may hold for speed is bounded by A or by 9 d n floats. Chunks shorter than
+// that cost their totals' traffic and a work item's start for few rows each: gather kernel, 50001 x 33,
+// d = 1056, FP32, R = 6256 / 2112 / 528: 39 / 60 / 106 us, tile kernel without totals 124 / 57 / 59; register
+// kernel, bfloat16, 2^20 x 64, d = 1024, k = 4, R = 2^17 / 4096 / 1024: 112 / 199 / 558 us, tile 220 / 234 / 353.
+bool chunks_pay_totals(const sk_plan_s* p, int64_t rows, int64_t R) {
+  const int64_t chunks = (p->row_offset % R + rows + R - 1) / R;
+  if (chunks > 9) return chunks <= rows / (4 * p->d);
+  return chunks == 1 || R >= 4096 || chunks * p->d <= rows;
+}
+
 // Owner-kernel configuration (atomic mode, SK_KERNEL_OWNER): blocks per item kb = 2 when two blocks
 // of 32-column lines fit in shared memory, else 1; false if the kernel does not apply.
 bool choose_own(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& di, bool tma_ok, TileCfg* cfg) {
@@ -274,9 +287,10 @@ bool choose_reg(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& di, 
     return false;
   }
   const size_t optin = (size_t)std::min(di.optin, 232448) - 1024;
+  const int64_t R = p->R > 0 ? p->R : default_chunk_rows(p->m);
+  if (a_type != SK_A_FP32 && !chunks_pay_totals(p, rows, R)) return false;
   int32_t nsub = 0, cap = 0;
   if (!reg_choose_box(p->d, p->B, a_type, optin, p->list_cap, &nsub, &cap)) return false;
-  const int64_t R = p->R > 0 ? p->R : default_chunk_rows(p->m);
   const int64_t ncg = (n + reg_cols(a_type) - 1) / reg_cols(a_type);
   const int64_t ntg = (p->d + reg_targets(a_type) - 1) / reg_targets(a_type);
   *cfg = TileCfg();
@@ -335,11 +349,12 @@ bool gather_wins(const sk_plan_s* p, int64_t n, int64_t rows, bool tma_ok, int32
 // here with 25 % allowed 1.34e-7).
 bool choose_gather(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& di, bool tma_ok, int32_t a_type,
                    TileCfg* cfg) {
+  const int64_t R = p->R > 0 ? p->R : default_chunk_rows(p->m);
   if (p->mode != SK_MODE_ATOMIC || p->kernel != SK_KERNEL_AUTO || p->tile_cols != 0 || p->threads != 0 ||
       !gather_wins(p, n, rows, tma_ok, a_type) ||
+      !chunks_pay_totals(p, rows, R) ||
       gat_smem_bytes(p->d, p->B, rows) > (size_t)std::min(di.optin, 232448) - 1024)
     return false;
-  const int64_t R = p->R > 0 ? p->R : default_chunk_rows(p->m);
   const int64_t ncg = (n + gat_cols() - 1) / gat_cols();
   const int64_t tgs = gat_targets(p->d), ntg = (p->d + tgs - 1) / tgs;
   const int64_t first = ((p->row_offset % R) + R) % R;

@@ -166,3 +166,19 @@ def test_eager_call_beside_another_streams_capture(sk, dev):
     assert np.array_equal(_bits(Z, 1), ref)
     first.close()
     plan.close()
+
+
+@pytest.mark.parametrize("R", [1, 7, 300])
+@pytest.mark.parametrize("a_type,k", [("float32", 1), ("bfloat16", 4)])
+def test_short_chunks(sk, dev, R, a_type, k):
+    import torch
+    m, n, d = 65536, 20 if a_type == "float32" else 64, 640
+    A = _ints(m, n, R)
+    plan = sk.Plan(d, m, k, 0, 11, chunk_rows=R)
+    Y = plan.apply(torch.from_numpy(A).to(dev).to(getattr(torch, a_type)))
+    torch.cuda.synchronize()
+    assert plan.get(sk.SK_PARAM_LAST_KERNEL) == sk.SK_KERNEL_TILE
+    assert plan.get(sk.SK_PARAM_SCRATCH_BYTES) <= 4 + BARRIER + 4 * m * n
+    # (k = 1 has scale 1 and integer sums, and k = 4 sums of halves: exact in any order)
+    assert np.array_equal(_bits(Y, 0), oracle.sketch_canonical(A, d, k, 11, 0, R))
+    plan.close()

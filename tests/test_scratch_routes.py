@@ -101,3 +101,19 @@ p = plan(WIDE); most.value = 0; assert apply(p, 257)[0] == GATHER; need = held(p
 p = plan(WIDE); most.value = need - 1
 assert apply(p, 257)[0] == GLOBAL and 4 < held(p) < 4 + need
 """)
+
+
+def test_short_chunks_need_no_large_totals(run):
+    # Totals are d x n floats for every chunk: with the chunk length of the paper's per-element scheme (1) they
+    # would be 17 TB here. What a plan holds for speed stays below A's own size in FP32.
+    run("""
+for R, t in ((1, 0), (1, 1), (7, 0), (64, 1), (256, 0), (1000, 1)):
+    p = sk.Plan(1024, 65536, 1 if t == 0 else 4, 1, 1, chunk_rows=R)
+    assert apply(p, 64, a_type=t)[0] == TILE and held(p) <= 4 + BAR + 4 * 65536 * 64, (R, t)
+p = sk.Plan(4096, 1 << 22, 1, 1, 1, chunk_rows=256)
+assert apply(p, 64)[0] == TILE and held(p) == 4
+for R, case, n, t, kern in ((0, GATH, 128, 0, GATHER), (8192, BOTH, 64, 0, TILE), (1 << 17, BOTH, 64, 0, GATHER),
+                            (2048, REG16, 64, 1, REG), (200, REG16, 64, 1, TILE)):
+    p = plan(case, chunk_rows=R)
+    assert apply(p, n, a_type=t)[0] == kern, (R, case)
+""")
