@@ -94,7 +94,8 @@ typedef enum {
    * k >= 2, n >= 32 and B = d/k <= 512 (except n >= 256 with k = 2) when A's layout allows TMA
    * (and neither SK_PARAM_TILE_COLS nor SK_PARAM_THREADS is set); the gather kernel (every output row has
    * one owner, which reads the rows of A that S sends to it; AUTO only) for most other sketches of at
-   * least 65536 rows, and of FP32 rows that TMA cannot read from 8192 to 32768 rows on; otherwise the
+   * least 65536 rows and d up to 8192, and of FP32 rows that TMA cannot read from 8192 to 131072 rows on,
+   * unless SK_PARAM_CHUNK_ROWS asks for chunks too short to pay for its totals; otherwise the
    * tile kernel, or the global kernel when a block of S is too tall for the tile kernel's shared-memory
    * accumulator, when the tile kernel would need several block groups or only 4-column items of a matrix
    * with n >= 256, and for n >= 256 at k <= 2. The register kernel for 16-bit A and the gather kernel need

@@ -307,37 +307,54 @@ bool choose_reg(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& di, 
   return true;
 }
 
-// Where AUTO takes the gather kernel, by where it was the fastest (n from 4 to 1024, d / n = 2, 8, 32,
-// k = 1, 2, 4, 8, 2^13 to 2^22 rows; in brackets the time of the kernel taken otherwise over its time):
-// - aligned rows, n < 256, from 65536 rows on (8192 with d >= 4096, n >= 64: 1.3 to 1.4; below that its fixed
-//   cost loses up to 30 %): k = 1 from 24 columns on (1.1 to 3.2; 16 columns use a quarter of its lanes and
-//   need 2^20 rows: 1.2); k = 2 below the register kernel's 32 columns (1.0 to 1.35); k >= 2 where blocks are
-//   too tall for that kernel, B > 512 (k = 2 1.25 to 1.8; k = 4 1.1 to 1.3, while a row's k reads waste few
-//   lanes: 0.96 at n = 100); d from 8192 to 16383, FP32 (2^22 x 64, k = 8: 1.4);
-// - FP32, n >= 256, from 131072 rows on: k <= 2 with n <= 512 and d <= 2048 (d <= 2 n 1.02 to 1.6; d above
-//   that from 2^20 rows on 1.13 to 1.3, at 131072 rows 0.85), k = 3 or 4 with B in (512, 1024] (2^19 x 1024:
-//   1.12); elsewhere the global kernel stays ahead (k = 8, d = 16384: 0.83);
-// - FP32 rows that TMA cannot read, from 32768 on: nearly everywhere (1.1 to 2.4; not with k = 8 and half of
-//   the last 64 columns empty, 0.88, nor with d above 8192 at k = 1); from 8192 on with k >= 2, n < 256 and d
-//   from 512 to 4224 (0.98 to 1.9).
+// Where AUTO takes the gather kernel: where it was the faster one of 16500 shapes (n from 17 to 4097, d up to 65536,
+// k = 1, 2, 3, 4, 8, 2^13 to 2^22 rows, default chunk length; over the 14500 inside the line 1.8 times as fast as
+// the kernel taken otherwise in the mean, 0.9 or less at 16). Every group of 512 output rows and every 64 columns
+// hash all rows again, so the cost grows with d n, and the rows have to pay for it. In brackets the time of the
+// other kernel over the gather kernel's beyond the line.
+// - Aligned rows, n < 256, from 65536 rows on (8192 with d >= 4096, n >= 64): k = 1 from 24 columns on, d up to
+//   8192; k = 2 below the register kernel's 32 columns (24 use 3/8 of the lanes: 0.73 at 2^22 rows, d = 4096);
+//   blocks too tall for that kernel, B > 512, while k reads of a row waste few lanes, or FP32 and d from 8192 to
+//   12288 (d = 14336: 0.7 to 0.9 below 2^20 rows). Not below 110000 rows with 129 to 159 columns (0.74 to 0.9) or
+//   k = 4 and more than 96 columns (0.82 to 0.94), both at d from 4096 to 8191; k = 4, d < 4096, n > 192: 0.77.
+// - FP32, n >= 256, from 131072 rows on: k <= 2 with n <= 512 and d <= 2048 (d = 2 n at 131072 rows: 0.81), k = 3 or 4
+//   with B in (512, 1024]; elsewhere the global kernel stays ahead.
+// - FP32 rows that TMA cannot read: d <= 8448 or a 128th of the rows (0.5 to 0.8 above); from 32768 rows on,
+//   with k >= 2, n < 256 and d from 512 to 4224 from 8192. k = 8 not with 40 % of the last 64 columns' lanes idle;
+//   k <= 2 later: an even n, for which the other kernel adds pairs (0.72 to 0.9 before), and k = 1 with few
+//   columns and output rows (0.84) or with n >= 256, where the global kernel makes few reductions (0.7 to 0.9).
 bool gather_wins(const sk_plan_s* p, int64_t n, int64_t rows, bool tma_ok, int32_t a_type) {
   const int64_t k = p->k, d = p->d, B = p->B, lanes = (n + 63) / 64 * 64;
   const bool f32 = a_type == SK_A_FP32;
   if (rows >= ((int64_t)1 << 31) || rows < 8192 || B < 64 || k > 8 || n < 16) return false;
   if (!tma_ok) {
-    if (!f32 || n < 17 || (k > 4 && 5 * n < 3 * lanes)) return false;
-    return rows >= 32768 ? k > 1 || d <= 8192 : k >= 2 && n < 256 && d >= 512 && d <= 4224;
+    if (!f32 || n < 17 || (k > 4 && 5 * n < 3 * lanes) || (d > 8448 && (k == 1 || rows < 128 * d))) return false;
+    if (n > 4100 || (n > 1024 && d > (k < 3 ? 2048 : 4096))) return false;
+    if (rows < 32768) return k >= 2 && n < 256 && d >= 512 && d <= 4224;
+    if (k == 2) {
+      if (n >= 256 && n < 384) return rows >= std::min<int64_t>(131072, std::max<int64_t>(50000, 128 * d));
+      return n % 2 != 0 || rows >= 50000;
+    }
+    if (k > 2 || d <= 128) return true;
+    if (n >= 512) return d <= 2048 || rows >= 32 * d;
+    if (n >= 256) return rows >= std::max<int64_t>(131072, 32 * d);
+    if (n % 2 == 0) return rows >= (d <= 2048 ? 65000 : 110000);
+    return rows >= 50000 || d >= 1024 || n >= 160;
   }
   if (n % 4 != 0 || (rows < 65536 && (d < 4096 || n < 64))) return false;
   if (n < 256) {
+    const bool mid = d >= 4096 && d < 8192;
+    if (n > 128 && n < 160 && mid && rows <= 110000) return false;
+    if (k == 4 && rows >= 24000 && rows < 110000 && ((n > 96 && mid) || (n > 192 && d < 4096 && rows < 80000))) return false;
     if (k == 1) return (n >= 24 || rows >= (1 << 20)) && d <= 8192;
-    if (n < 32) return k == 2 && n >= 24;
+    if (n < 32) return k == 2 && n >= 24 && d <= 8192 && (rows <= (1 << 20) || d <= (n < 28 ? 512 : 4096));
     if (B <= 512 || n < 48) return false;
-    return k * lanes <= 5 * n ? d <= 8192 : f32 && d >= 8192 && d < 16384;
+    if (k * lanes <= 5 * n) return d <= 8192;
+    return f32 && d >= 8192 && d < 16384 && (d <= 12288 || (n <= 64 && rows >= (1 << 20)));
   }
   if (!f32 || rows < 131072) return false;
-  if (k <= 2) return n <= 512 && d <= 2048 && (d <= 2 * n || rows >= (1 << 20));
-  return k <= 4 && B > 512 && B <= 1024;
+  if (k <= 2) return n <= 512 && d <= 2048 && (d <= n || (d <= 2 * n && rows >= (1 << 18)) || rows >= (1 << 20));
+  return k <= 4 && n <= 2048 && B > 512 && B <= 1024;
 }
 
 // Gather-kernel configuration. The slices are the ones for which the rounds of work items end first, an item

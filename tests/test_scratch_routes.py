@@ -96,7 +96,7 @@ most.value = 1 << 15  # cudaMalloc of more than this fails
 for case, n, t in ((SMALL, 16, 0), (GATH, 128, 0), (REG16, 64, 1)):
     p = plan(case)
     assert apply(p, n, a_type=t) == (TILE, 0, 1) and held(p) == 4
-WIDE = dict(d=8192, m=65536, k=2), 257  # gather kernel, else the global kernel, in passes with smaller totals
+WIDE = dict(d=8190, m=65536, k=3), 257  # gather kernel, else the global kernel, in passes with smaller totals
 p = plan(WIDE); most.value = 0; assert apply(p, 257)[0] == GATHER; need = held(p) - 4
 p = plan(WIDE); most.value = need - 1
 assert apply(p, 257)[0] == GLOBAL and 4 < held(p) < 4 + need
@@ -116,4 +116,19 @@ for R, case, n, t, kern in ((0, GATH, 128, 0, GATHER), (8192, BOTH, 64, 0, TILE)
                             (2048, REG16, 64, 1, REG), (200, REG16, 64, 1, TILE)):
     p = plan(case, chunk_rows=R)
     assert apply(p, n, a_type=t)[0] == kern, (R, case)
+""")
+
+
+def test_gather_kernel_leaves_tall_sketches_to_others(run):
+    # The gather kernel's work grows with d n; the kernels taken otherwise make k n additions a row whatever d.
+    run("""
+for d, m, k, n, want in ((32768, 1 << 20, 2, 33, False), (262144, 1 << 20, 2, 33, False), (1 << 20, 1 << 20, 8, 33, False),
+                         (16384, 1 << 18, 4, 65, False), (16384, 1 << 22, 4, 65, True), (8192, 32768, 4, 33, True),
+                         (65536, 1 << 20, 2, 28, False), (2048, 1 << 20, 2, 28, True), (4096, 1 << 22, 2, 24, False),
+                         (15000, 1 << 17, 4, 100, False), (8192, 1 << 17, 4, 100, True), (1024, 1 << 17, 1, 512, False),
+                         (1024, 1 << 19, 1, 512, True), (4096, 40000, 4, 128, False), (4096, 1 << 17, 4, 128, True),
+                         (8192, 1 << 17, 3, 1537, False), (4096, 1 << 17, 3, 1537, True), (1024, 40000, 3, 5001, False),
+                         (2048, 65536, 1, 257, False), (2048, 1 << 18, 1, 257, True), (2048, 40000, 1, 130, False)):
+    p = sk.Plan(d // k * k, m, k, 1, 1)
+    assert (apply(p, n)[0] == GATHER) == want, (d, m, k, n)
 """)
