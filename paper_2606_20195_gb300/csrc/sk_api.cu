@@ -119,18 +119,38 @@ size_t plan_scratch_bytes(const sk_plan_s* p) {
          2 * p->stage_bytes + p->ydev_bytes;
 }
 
+// Give back the chunk totals that the plan's sketches can do without (cudaFree waits for their users).
+bool drop_fast(sk_plan_s* p) {
+  if (!p->fastP) return false;
+  cudaFree(p->fastP);
+  p->fastP = nullptr;
+  p->fastP_bytes = 0;
+  return true;
+}
+
+// Whether `bytes` more of scratch in place of `cur` fit the plan's limit, if need be after giving back the
+// totals that its sketches can do without.
+bool fits_limit(sk_plan_s* p, size_t cur, size_t bytes) {
+  if (p->scratch_limit <= 0) return true;
+  const size_t limit = (size_t)p->scratch_limit, others = plan_scratch_bytes(p) - cur + bytes;
+  if (others <= limit) return true;
+  return others - p->fastP_bytes <= limit && drop_fast(p);
+}
+
 // Replace one plan buffer (*ptr of *cur bytes) by a new one of `bytes`: checked against the plan's
 // scratch limit first, so a refused call leaves the plan's buffers as they were and enqueues nothing;
 // SK_ERR_OOM also when cudaMalloc fails.
 template <typename T>
 sk_status plan_grow(sk_plan_s* p, T** ptr, size_t* cur, size_t bytes, const char* what) {
-  if (p->scratch_limit > 0 && plan_scratch_bytes(p) - *cur + bytes > (size_t)p->scratch_limit)
+  if (!fits_limit(p, *cur, bytes))
     return set_error(SK_ERR_OOM, "%s (%zu bytes) would take the plan's scratch above its limit of %lld bytes", what,
                      bytes, (long long)p->scratch_limit);
   if (*ptr) cudaFree(*ptr);
   *ptr = nullptr;
   *cur = 0;
-  if (cudaMalloc(reinterpret_cast<void**>(ptr), bytes) != cudaSuccess) {
+  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(ptr), bytes);
+  if (e != cudaSuccess && drop_fast(p)) e = cudaMalloc(reinterpret_cast<void**>(ptr), bytes);
+  if (e != cudaSuccess) {
     cudaGetLastError();
     return set_error(SK_ERR_OOM, "%s (%zu bytes)", what, bytes);
   }
@@ -984,7 +1004,7 @@ sk_status sk_apply_host(sk_plan p, const float* A_host, int64_t lda, int64_t n, 
   const size_t ybytes = elem_size(p->rule) * (size_t)(p->d * n);
   if (p->stage_bytes < tile_bytes) {
     // both staging tiles at once against the limit (plan_grow counts stage_bytes twice)
-    if (p->scratch_limit > 0 && plan_scratch_bytes(p) - 2 * p->stage_bytes + 2 * tile_bytes > (size_t)p->scratch_limit)
+    if (!fits_limit(p, 2 * p->stage_bytes, 2 * tile_bytes))
       return set_error(SK_ERR_OOM, "host pipeline staging (2 x %zu bytes) would take the plan's scratch above its limit",
                        tile_bytes);
     for (int b = 0; b < 2; ++b) {
@@ -993,7 +1013,8 @@ sk_status sk_apply_host(sk_plan p, const float* A_host, int64_t lda, int64_t n, 
     }
     p->stage_bytes = 0;
     for (int b = 0; b < 2; ++b) {
-      if (cudaMalloc(&p->stage[b], tile_bytes) != cudaSuccess) {
+      if (cudaMalloc(&p->stage[b], tile_bytes) != cudaSuccess &&
+          (!drop_fast(p) || cudaMalloc(&p->stage[b], tile_bytes) != cudaSuccess)) {
         cudaGetLastError();
         return set_error(SK_ERR_OOM, "host pipeline staging (%zu bytes)", tile_bytes);
       }

@@ -45,6 +45,9 @@ int cudaMemcpyAsync(void* d, const void* s, size_t n, int kind, void* st) {
 int cudaMemcpy(void* d, const void* s, size_t n, int kind) { return cudaMemcpyAsync(d, s, n, kind, 0); }
 int cudaStreamIsCapturing(void* st, int* status) { return (void)st, *status = fake_capturing, OK; }
 int cudaStreamGetId(void* st, unsigned long long* id) { return *id = (unsigned long long)(size_t)st, OK; }
+int cudaStreamCreateWithFlags(void** st, unsigned fl) { return (void)fl, *st = malloc(8), OK; }
+int cudaStreamDestroy(void* st) { return free(st), OK; }
+int cudaStreamWaitEvent(void* st, void* e, unsigned fl) { return (void)st, (void)e, (void)fl, OK; }
 int cudaThreadExchangeStreamCaptureMode(int* mode) { return (void)mode, OK; }
 int cudaEventCreateWithFlags(void** e, unsigned fl) { return (void)fl, *e = malloc(8), OK; }
 int cudaEventDestroy(void* e) { return free(e), OK; }

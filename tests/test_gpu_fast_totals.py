@@ -182,3 +182,23 @@ def test_short_chunks(sk, dev, R, a_type, k):
     # (k = 1 has scale 1 and integer sums, and k = 4 sums of halves: exact in any order)
     assert np.array_equal(_bits(Y, 0), oracle.sketch_canonical(A, d, k, 11, 0, R))
     plan.close()
+
+
+def test_apply_then_solve_under_the_solves_limit(sk, dev):
+    import torch
+    m, n, d, k = 16384, 16, 256, 4
+    A = _ints(m, n, 5)
+    Ad, Y = torch.from_numpy(A).to(dev), torch.empty((d, n), device=dev)
+    b = torch.from_numpy(A @ np.arange(1.0, n + 1, dtype=np.float32)).to(dev)
+    alone, plan = sk.Plan(d, m, k, 0, 11), sk.Plan(d, m, k, 0, 11)
+    sk.sk_solve_sketched(alone.handle, torch.zeros((d, n + 1), device=dev), n + 1, n, torch.empty(n, device=dev))
+    plan.apply(Ad, Y)
+    plan.set(sk.SK_PARAM_SCRATCH_LIMIT, alone.get(sk.SK_PARAM_SCRATCH_BYTES) + 4)
+    x = plan.solve(Ad, b)  # A x = b holds exactly, so the sketched solution is 1 .. n
+    assert plan.solve_status()[0] == 0
+    assert np.allclose(x.cpu().numpy(), np.arange(1, n + 1), rtol=1e-5)
+    plan.apply(Ad, Y)
+    torch.cuda.synchronize()
+    assert np.array_equal(_bits(Y, 0), oracle.sketch_canonical(A, d, k, 11, 0, plan.get(sk.SK_PARAM_LAST_CHUNK_ROWS)))
+    alone.close()
+    plan.close()

@@ -132,3 +132,28 @@ for d, m, k, n, want in ((32768, 1 << 20, 2, 33, False), (262144, 1 << 20, 2, 33
     p = sk.Plan(d // k * k, m, k, 1, 1)
     assert (apply(p, n)[0] == GATHER) == want, (d, m, k, n)
 """)
+
+
+def test_optional_totals_are_given_back(run):
+    # The totals a sketch can do without must not stand in the way of scratch that a later call needs: under the
+    # limit that sk_solve or sk_apply_host needs by itself, and where the device's memory is short.
+    run("""
+for case, n in ((SMALL, 16), (GATH, 128)):
+    alone = plan(case)
+    sk.sk_solve_sketched(alone.handle, Y, n + 1, n, Y, ST); need = held(alone)
+    p = plan(case)
+    fast = apply(p, n)
+    p.set(sk.SK_PARAM_SCRATCH_LIMIT, need + 4 + 1000)  # room for the solve's scratch, not for both
+    f0 = frees.value
+    sk.sk_solve(p.handle, A, n, n, A, Y, ST)
+    assert held(p) <= need + 4 and frees.value == f0 + 1
+    assert apply(p, n) == (TILE, 0, 1) and held(p) == need + 4
+    p.set(sk.SK_PARAM_SCRATCH_LIMIT, 0)
+    assert apply(p, n) == fast
+    p = plan(case); apply(p, n)
+    tile = 4 * case[0]["m"] * n; y = 2 * case[0]["d"] * n
+    p.set(sk.SK_PARAM_SCRATCH_LIMIT, 4 + 2 * tile + y)
+    out = ctypes.create_string_buffer(y)
+    sk.sk_apply_host(p.handle, A, n, n, ctypes.addressof(out), ST)
+    assert held(p) == 4 + 2 * tile + y
+""")
