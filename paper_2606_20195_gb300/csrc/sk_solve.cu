@@ -241,7 +241,9 @@ __device__ void back_substitute(const SolveLaunch& L, double* rhs) {
   }
   if (tid == 0) {
     if (singular) atomicOr(L.status, kStatusNumeric);
-    *L.kappa = (rmin > 0.0) ? rmax / rmin : __longlong_as_double(0x7ff0000000000000ll);
+    // (fmax and fmin drop NaN: with nothing but NaN on the diagonal rmax is still 0 and rmin infinite)
+    const double inf = __longlong_as_double(0x7ff0000000000000ll);
+    *L.kappa = (rmin > 0.0 && rmin <= rmax && rmax < inf) ? rmax / rmin : inf;
   }
 }
 
