@@ -252,8 +252,14 @@ __device__ void back_substitute(const SolveLaunch& L, double* rhs) {
   }
 }
 
-template <typename T, int NB>
-__global__ void __launch_bounds__(kQRThreads) qr64_kernel(const QRArgs a) {
+// CTAS: CTAs that an SM's registers are to have room for. A wide sketch takes most of an SM's shared memory per
+// CTA, and its CTAs all the registers they can use. A narrow one has to leave room: its cooperative launch
+// starts when every CTA has a place, and a CTA with 255 registers a thread has none beside another request's
+// kernel. A service's saturated stream of requests (n up to 256; m from 2^14 to 2^24, or to 2^20 rows) then
+// makes 363 / 1290 solves a second, with 128 registers 381 / 1530 (384 / 1360 with the kernel that took one
+// reduction per column and 64 registers). One QR alone takes 1 to 2 % longer: 1024 x 64 279 us, not 275.
+template <typename T, int NB, int CTAS>
+__global__ void __launch_bounds__(kQRThreads, CTAS) qr64_kernel(const QRArgs a) {
   const long long wait = a.L.wait_cycles > 0 ? a.L.wait_cycles : kBarrierCycles;
   extern __shared__ __align__(16) double Wl[];  // rpc x (n+1) rows of W (row-major)
   __shared__ double wsm[NB * NB], rsm[NB * NB], lsm[NB * NB], taus[NB], v0s[NB];
@@ -458,12 +464,12 @@ int32_t solve_ctas(int64_t d, int64_t n, int32_t sms, size_t smem_optin) {
 }
 
 // The kernel for an element type and panel width.
-template <int NB>
+template <int NB, int CTAS>
 static const void* qr_kernel(const SolveLaunch& L) {
-  if (L.src_fp64) return (const void*)qr64_kernel<double, NB>;
-  if (L.rule == kFP32) return (const void*)qr64_kernel<float, NB>;
-  if (L.rule == kBF16) return (const void*)qr64_kernel<__nv_bfloat16, NB>;
-  return (const void*)qr64_kernel<__half, NB>;
+  if (L.src_fp64) return (const void*)qr64_kernel<double, NB, CTAS>;
+  if (L.rule == kFP32) return (const void*)qr64_kernel<float, NB, CTAS>;
+  if (L.rule == kBF16) return (const void*)qr64_kernel<__nv_bfloat16, NB, CTAS>;
+  return (const void*)qr64_kernel<__half, NB, CTAS>;
 }
 
 cudaError_t launch_solve(const SolveLaunch& L, cudaStream_t st, int32_t* launches) {
@@ -482,7 +488,10 @@ cudaError_t launch_solve(const SolveLaunch& L, cudaStream_t st, int32_t* launche
   if (e != cudaSuccess) return e;
   const size_t smem = std::max<size_t>((size_t)a.rpc * (size_t)(L.n + 1) * 8, (size_t)L.n * 8);
   void* args[] = {(void*)&a};
-  const void* kern = nb == 16 ? qr_kernel<16>(L) : nb == 8 ? qr_kernel<8>(L) : qr_kernel<4>(L);
+  const bool alone = 2 * smem > 200 * 1024;  // no second CTA of this size on an SM
+  const void* kern = nb == 16 ? (alone ? qr_kernel<16, 1>(L) : qr_kernel<16, 2>(L))
+                     : nb == 8 ? qr_kernel<8, 2>(L)
+                               : qr_kernel<4, 2>(L);
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   e = cudaLaunchCooperativeKernel(kern, dim3((unsigned)L.ncta), dim3(kQRThreads), args, smem, st);
