@@ -276,7 +276,8 @@ SK_API sk_status sk_solve_status(sk_plan plan, double* kappa, void* stream);
  *   max_iters: iteration limit (<= 0: 100). tol: stop when the estimate of
  *     ||(A R^{-1})^T r|| / (||A R^{-1}||_F ||r||) <= tol or ||r|| <= tol ||b - A x0|| (<= 0: 1e-10).
  *   iters_out (may be NULL): iterations used.
- * Every iteration runs on the GPU in FP64; the call synchronizes `stream` every few iterations to
+ * Every iteration runs on the GPU: products with A and the m-vector u in pairs of floats (about 48
+ * bits), the n-vectors and scalars in FP64. The call synchronizes `stream` every few iterations to
  * test convergence and returns when x_dev is written. Scratch (m + 9n doubles) is plan-owned.
  * Errors: as sk_solve; SK_ERR_NUMERIC if S A is rank deficient (no preconditioner).
  */

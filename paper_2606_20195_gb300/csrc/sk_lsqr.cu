@@ -69,6 +69,16 @@ __device__ __forceinline__ void df_add(float& s, float& c, float s2, float c2) {
   c = __fadd_rn(__fadd_rn(c, c2), err);
 }
 
+// c = (hi + lo) * scale with hi of magnitude 1/2 to 1 and scale a power of two (2^-120 to 2^120): lo keeps its
+// bits whatever c's exponent, where the second float of c itself would be subnormal from about 1e-31 down.
+__device__ __forceinline__ void split_scaled(double c, float& hi, float& lo, float& scale) {
+  int e = 0;
+  const double f = frexp(c, &e);
+  const int es = max(-120, min(120, e));
+  split_df(ldexp(f, e - es), hi, lo);
+  scale = __uint_as_float((uint32_t)(es + 127) << 23);
+}
+
 constexpr int kPassThreads = 256;
 constexpr int kPassCols = 16;  // columns per lane
 constexpr int kPassDepth = 4;  // row groups in flight per warp, one of them being used
@@ -99,7 +109,9 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src, bool ok) {
 // Bounds: the bytes of A (once) and, close behind, the FP32 pipe: df_acc2 is 12 operations, twice
 // per pair of elements. The partial dot products are combined over the LPR lanes and c u is added in float pairs:
 // on this GPU an FP64 operation takes a warp 16 cycles of the SM's FP64 pipe, and here it would be
-// repeated by the LPR lanes of a row. Rows arrive through a per-thread cp.async ring: with the next row
+// repeated by the LPR lanes of a row. That is no less exact than a lane's row-long float-pair sum followed by an
+// FP64 combination: x off by 1.3e-16 at 2^18 x 128 (7.6e-16 with the latter), 5.8e-16 at 65536 x 512 (1.2e-14),
+// 1.3e-13 at 2^18 x 100 with column scales from 1 to 1e-3 (2.4e-13). Rows arrive through a per-thread cp.async ring: with the next row
 // prefetched into registers only, 336 us, the loads' latency exposed. The FP64 sum of u^2 takes one lane per row: the lanes of a row
 // keep the u of LPR successive rows, then all 32 add theirs. Measured on GB300 at 2^21 x 128: 303 us
 // against 327 us (A p) + 295 us (A^T u) in two passes.
@@ -122,8 +134,8 @@ __global__ void __launch_bounds__(kPassThreads, 2) lsqr_pass_kernel(const LsqrLa
     zs[j] = 0.0;
   }
   __syncthreads();
-  float ch = 0.f, cl = 0.f;
-  if (!b) split_df(L.sc[kLsqrC], ch, cl);
+  float ch = 0.f, cl = 0.f, cscale = 1.f;
+  if (!b) split_scaled(L.sc[kLsqrC], ch, cl, cscale);
   float* uh = reinterpret_cast<float*>(L.u);
   float* ul = uh + m;
   // Column of this lane's element q: whole float4 chunks (VEC) or single floats, interleaved over the
@@ -170,7 +182,7 @@ __global__ void __launch_bounds__(kPassThreads, 2) lsqr_pass_kernel(const LsqrLa
       a[q + 2] = v.z;
       a[q + 3] = v.w;
     }
-    const float oh = S.uh[tid], ol = S.ul[tid];
+    const float oh = cscale * S.uh[tid], ol = cscale * S.ul[tid];  // (exact; cscale is 1 where these are b)
     const bool live = row < m;
     float2 s2 = make_float2(0.f, 0.f), c2 = make_float2(0.f, 0.f);
     if constexpr (VEC) {
