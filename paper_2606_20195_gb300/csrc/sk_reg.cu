@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(RegShape<AT>::kThreads, 1) reg_kernel(const Re
 #pragma unroll 1
         for (; la != le; la += 2u * threads) {
           int32_t e;  // sign-extended: the sign of the entry is the sign of the register
-          asm volatile("ld.shared.s16 %0, [%1];" : "=r"(e) : "r"(la));
+          asm volatile("ld.shared.s16 %0, [%1];" : "=r"(e) : "r"(la) : "memory");
           const uint32_t ra = rows + (((uint32_t)e & 0x7FFFu) << 7);
           const float sg = __uint_as_float(((uint32_t)e & 0x80000000u) | 0x3F800000u);
 #pragma unroll
@@ -342,7 +342,8 @@ __global__ void __launch_bounds__(RegShape<AT>::kThreads, 1) reg_kernel(const Re
             uint4 v;
             asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
                          : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                         : "r"(ra ^ ((uint32_t)q << 4)));
+                         : "r"(ra ^ ((uint32_t)q << 4))
+                         : "memory");
             reg_add<AT>(v, sg, acc[q]);
           }
         }
