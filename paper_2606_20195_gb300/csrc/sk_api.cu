@@ -224,12 +224,18 @@ int32_t choose_slices(const sk_plan_s* p, int64_t rows, int64_t R, int64_t ncg, 
 // (and, but for the register kernel, one launch that finishes the chunk totals itself): 16384 x 16,
 // d = 256, k = 4 (4 items / 152): 42 / 14.5 us; 50001 x 33, d = 1056, k = 4 (16 / 144): 175 / 55;
 // 65536 x 64, d = 1024, k = 4 (32 / 144, register kernel): 47 / 28; 8192 x 64, d = 8192, k = 4: 43 / 28.
+// Where half of the CTAs make slices of up to 320 rows, half it is: alone such a call is as fast, and two run side
+// by side (30 plans on 30 streams, us a call: 16384 x 16 11.5 -> 6.2, one slice a chunk 7.0; 3000 x 12, d = 4096,
+// k = 2 14.9 -> 7.9 and 6.7). Larger ones lose beside others part of what they gain alone: 65536 x 64 48 -> 29
+// alone, 8.5 -> 13.3 beside 29 others; 60000 x 20, d = 320, k = 8 201 -> 27 and 12 -> 25.
 int32_t fill_slices(const sk_plan_s* p, int64_t n, int64_t rows, int64_t R, int64_t ncg, int64_t nbg, int32_t cps,
                     const DevInfo& di, int32_t slices, bool finishes) {
   const int64_t first = ((p->row_offset % R) + R) % R;
   const int64_t per = (first + rows + R - 1) / R * ncg * nbg;
   const int64_t chunk = std::min(R, rows);
   int64_t fit = std::min((int64_t)di.sms * std::max(cps, 1) / per, std::max<int64_t>(1, chunk / 64));
+  const int64_t half = (int64_t)di.sms * std::max(cps, 1) / (2 * per);
+  if (half >= 3 && chunk <= 320 * half) fit = std::min(fit, half);
   if (n % 4 != 0) fit = std::min(fit, chunk * p->k / p->d);
   if (fit <= slices || (!finishes && slices == 1 && fit < 3)) return slices;
   return (int32_t)fit;

@@ -22,13 +22,22 @@ int cudaDeviceGetAttribute(int* v, int attr, int dev) {
 int cudaFuncSetAttribute(const void* f, int a, int v) { return (void)f, (void)a, (void)v, OK; }
 int cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void* f, int threads, size_t smem, unsigned fl) {
   (void)f, (void)fl;
-  int by_threads = 2048 / threads, by_smem = smem ? (int)(233472 / (smem + 1024)) : 32;
+  /* 64 registers a thread */
+  int by_threads = 1024 / threads, by_smem = smem ? (int)(233472 / (smem + 1024)) : 32;
   *n = by_threads < by_smem ? by_threads : by_smem;
   return OK;
 }
 int __cudaGetKernel(void** k, const void* f) { return *k = (void*)f, OK; }
 int __cudaLaunchKernel(void* k, ...) { return (void)k, ++fake_kernels, OK; }
-int cudaLaunchCooperativeKernel(const void* k, ...) { return (void)k, ++fake_coop, OK; }
+typedef struct {
+  unsigned x, y, z;
+} dim3;
+unsigned fake_grid = 0; /* CTAs of the last cooperative launch */
+int cudaLaunchCooperativeKernel(const void* k, dim3 grid, dim3 block, void** args, size_t smem, void* st) {
+  (void)k, (void)block, (void)args, (void)smem, (void)st;
+  fake_grid = grid.x;
+  return ++fake_coop, OK;
+}
 int cudaMalloc(void** p, size_t bytes) {
   if (fake_max && bytes > fake_max) return OOM;
   ++fake_mallocs;

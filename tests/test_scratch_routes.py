@@ -157,3 +157,16 @@ for case, n in ((SMALL, 16), (GATH, 128)):
     sk.sk_apply_host(p.handle, A, n, n, ctypes.addressof(out), ST)
     assert held(p) == 4 + 2 * tile + y
 """)
+
+
+def test_small_sketches_leave_room_beside_them(run):
+    # A one-launch sketch waits at a grid barrier, so its CTAs must all be resident: over half of the GPU's 152, two
+    # calls on two streams run one after the other. Small ones are as fast on half of them.
+    run("""
+grid = var("fake_grid", ctypes.c_uint)
+for (m, n, d, k), half in (((16384, 16, 256, 4), True), ((20000, 1, 256, 4), True), ((3000, 12, 4096, 2), True),
+                           ((60000, 20, 320, 8), False), ((30000, 32, 1024, 1), False)):
+    p = sk.Plan(d, m, k, 1, 1)
+    assert apply(p, n) == (TILE, 1, 0)
+    assert (grid.value <= 76) == half and grid.value >= 38, (m, n, grid.value)
+""")
