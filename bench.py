@@ -90,6 +90,11 @@ def measured_peaks() -> dict:
     return {}
 
 
+# CUDA kernel by its number in SK_PARAM_LAST_KERNEL.
+KERNEL_NAMES = {1: "tile_kernel", 2: "literal_kernel", 3: "own_kernel", 4: "global_kernel", 5: "det_kernel",
+                6: "reg_kernel", 7: "gather_kernel"}
+
+
 def traffic_record(kernel: str, workload: str, rule: str):
     """DRAM traffic per launch from the committed ncu summary, if it was taken on these sources."""
     p = os.path.join(HERE, "profiles", f"{kernel}_{workload}_{rule}_traffic.txt")
@@ -819,9 +824,7 @@ def main() -> int:
     clocks = clk.summary()
     launches_per_step = plan.get(sk.SK_PARAM_LAST_LAUNCHES)
     R_used = plan.get(sk.SK_PARAM_LAST_CHUNK_ROWS)
-    kernel_name = {sk.SK_KERNEL_TILE: "tile_kernel", sk.SK_KERNEL_OWNER: "own_kernel",
-                   sk.SK_KERNEL_LITERAL: "literal_kernel", sk.SK_KERNEL_GLOBAL: "global_kernel",
-                   sk.SK_KERNEL_REGISTER: "reg_kernel"}.get(plan.get(sk.SK_PARAM_LAST_KERNEL), "det_kernel")
+    kernel_name = KERNEL_NAMES[plan.get(sk.SK_PARAM_LAST_KERNEL)]
     t = torch.tensor([total_ms], device=dev)
     if world > 1:
         dist.all_reduce(t, op=dist.ReduceOp.MAX)

@@ -115,7 +115,7 @@ typedef enum {
   SK_PARAM_DEVICE_STATUS = 9,
   /* Read-only: the kernel the last sketch ran: SK_KERNEL_TILE (1), SK_KERNEL_LITERAL (2),
    * SK_KERNEL_OWNER (3), SK_KERNEL_GLOBAL (4), 5 for the deterministic-mode kernel, or
-   * SK_KERNEL_REGISTER (6), 7 for the gather kernel (chunk accumulation by output rows, each row of A
+   * SK_KERNEL_REGISTER (6), SK_KERNEL_GATHER (7: chunk accumulation by output rows, each row of A
    * read by the owners of its target rows; AUTO only); 0 before the first sketch. */
   SK_PARAM_LAST_KERNEL = 10,
   /* Rows per group of sk_solve's tree QR (0, the default: as many rows as the GPU's shared memory
@@ -161,7 +161,8 @@ enum {
   SK_KERNEL_OWNER = 3,
   SK_KERNEL_GLOBAL = 4,
   /* 5 is the deterministic-mode kernel's number in SK_PARAM_LAST_KERNEL; it cannot be requested. */
-  SK_KERNEL_REGISTER = 6
+  SK_KERNEL_REGISTER = 6,
+  SK_KERNEL_GATHER = 7 /* in SK_PARAM_LAST_KERNEL; AUTO takes it, it cannot be requested */
 };
 
 typedef struct sk_plan_s* sk_plan;

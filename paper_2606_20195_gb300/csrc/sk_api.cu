@@ -814,7 +814,7 @@ sk_status enqueue_sketch(sk_plan_s* p, const void* A, int64_t lda, int64_t n, in
                         : cfg.reg ? "register kernel launch"
                         : cfg.own ? "owner kernel launch"
                                   : "tile kernel launch");
-  p->last_kernel = cfg.gat ? kGatherKernel : cfg.glob ? SK_KERNEL_GLOBAL : cfg.reg ? SK_KERNEL_REGISTER : cfg.own ? SK_KERNEL_OWNER : SK_KERNEL_TILE;
+  p->last_kernel = cfg.gat ? SK_KERNEL_GATHER : cfg.glob ? SK_KERNEL_GLOBAL : cfg.reg ? SK_KERNEL_REGISTER : cfg.own ? SK_KERNEL_OWNER : SK_KERNEL_TILE;
   if (R_used) *R_used = cfg.R;
   return SK_OK;
 }
@@ -1439,7 +1439,7 @@ sk_status sk_apply_partials(sk_plan p, const float* A, int64_t lda, int64_t n, f
   p->last_noalloc = false;
   p->last_launches = launches;
   p->last_R = R;
-  p->last_kernel = cfg.gat ? kGatherKernel : cfg.reg ? SK_KERNEL_REGISTER : cfg.own ? SK_KERNEL_OWNER : SK_KERNEL_TILE;
+  p->last_kernel = cfg.gat ? SK_KERNEL_GATHER : cfg.reg ? SK_KERNEL_REGISTER : cfg.own ? SK_KERNEL_OWNER : SK_KERNEL_TILE;
   return SK_OK;
 }
 

@@ -8,8 +8,6 @@ namespace sk {
 
 struct TileDesc;
 
-constexpr int32_t kGatherKernel = 7;  // its number in SK_PARAM_LAST_KERNEL
-
 struct TileLaunch {
   const void* A;    // elements of type a_type (0 FP32, 1 binary16, 2 bfloat16)
   int32_t a_type = 0;

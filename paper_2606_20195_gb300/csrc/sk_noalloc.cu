@@ -69,7 +69,7 @@ extern "C" SK_API sk_status sk_apply_noalloc(sk_plan p, const float* A, int64_t 
   e = launch_tile(L, st, &launches);
   if (e != cudaSuccess) return set_error(SK_ERR_CUDA, "sketch kernel launch: %s", cudaGetErrorString(e));
   noalloc_record(p, launches, L.R,
-                 L.gat ? kGatherKernel : L.glob ? SK_KERNEL_GLOBAL : L.reg ? SK_KERNEL_REGISTER : L.own ? SK_KERNEL_OWNER : SK_KERNEL_TILE);
+                 L.gat ? SK_KERNEL_GATHER : L.glob ? SK_KERNEL_GLOBAL : L.reg ? SK_KERNEL_REGISTER : L.own ? SK_KERNEL_OWNER : SK_KERNEL_TILE);
   return SK_OK;
 }
 

@@ -23,7 +23,7 @@ SK_PARAM_SCRATCH_LIMIT, SK_PARAM_SOLVE_WAIT_CYCLES, SK_PARAM_SCRATCH_BYTES, SK_P
 SK_PARAM_ITEM_CHUNKS = 17
 SK_MODE_ATOMIC, SK_MODE_DETERMINISTIC, SK_MODE_SERIAL_TILE = 0, 1, 2
 SK_KERNEL_AUTO, SK_KERNEL_TILE, SK_KERNEL_LITERAL, SK_KERNEL_OWNER, SK_KERNEL_GLOBAL = 0, 1, 2, 3, 4
-SK_KERNEL_REGISTER = 6
+SK_KERNEL_REGISTER, SK_KERNEL_GATHER = 6, 7
 SK_A_FP32, SK_A_FP16, SK_A_BF16 = 0, 1, 2
 
 # Every symbol include/sk.h declares.

@@ -41,3 +41,18 @@ def test_coherence_extremes():
     # a basis with every row of equal norm n/m has coherence 1
     H = np.kron(np.eye(n), np.ones((m // n, 1))) / np.sqrt(m // n)
     assert bench.coherence_of(torch.from_numpy(H)) == pytest.approx(1.0)
+
+
+def test_every_kernel_has_its_name():
+    # the bench line names the kernel that ran by its number; each name is a kernel of the sources
+    import glob
+    import os
+    import re
+
+    from bench import KERNEL_NAMES
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    header = open(os.path.join(root, "include", "sk.h")).read()
+    numbers = {int(v) for v in re.findall(r"\bSK_KERNEL_\w+\s*=\s*(\d+)", header)} - {0} | {5}
+    assert set(KERNEL_NAMES) == numbers
+    src = "".join(open(f).read() for f in glob.glob(os.path.join(root, "paper_2606_20195_gb300", "csrc", "*.cu*")))
+    assert all(re.search(r"\b%s\(" % name, src) for name in KERNEL_NAMES.values())
