@@ -299,8 +299,8 @@ void choose_global(const sk_plan_s* p, TileCfg* cfg) {
 // capacity for the plan's block height, the default chunk length and the slice count. AUTO takes it
 // for k >= 2, n >= 32 and blocks of at most 512 rows (not n >= 256 with k = 2, which goes to the
 // global kernel), where it is faster than the tile kernel
-// (measured at 2^22 x 64: d = 4096, k = 8: 1060 vs 818 GB/s; d = 1024, k = 8: 1520 vs 798; at
-// d = 4096 with k = 4 or 2 (B = 1024, 2048) the tile kernel stays ahead: 1416 vs 1357, 1735 vs 1448;
+// (measured at 2^22 x 64: d = 4096, k = 8: 1060 vs 818 GB/s; d = 1024, k = 8: 1520 vs 798; taller blocks, as
+// d = 4096 with k = 4 or 2, are the gather kernel's: 582 and 369 us, tile kernel 759 and 618, this one 791 and 741;
 // bfloat16 A: d = 4096, k = 8: 732 vs 1332 us; d = 1024, k = 4: 287 vs 735; 2^21 x 40, d = 320, k = 4:
 // 162 vs 356; 20000 x 128, d = 2048, k = 4: 26 vs 34; 2^18 x 1024, d = 2048, k = 4: 546 vs 917).
 bool choose_reg(const sk_plan_s* p, int64_t n, int64_t rows, const DevInfo& di, bool tma_ok, int32_t a_type,

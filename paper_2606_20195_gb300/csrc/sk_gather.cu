@@ -23,7 +23,8 @@
 //      lists, and a warp waits only for the longer of two.
 // Lists and counters are double-buffered: in the phase between two barriers half of the warps hash the next
 // box before they fetch and half after, so that hashing and memory latency overlap.
-// What bounds it: at k = 1 the loads in flight (64 KB a CTA; 4.1 TB/s at 2^22 x 64), at k = 4 the L1 data path
+// What bounds it: at k = 1 the loads in flight (at most 128 KB a CTA, and half of its warps hash meanwhile; 4.1
+// TB/s at 2^22 x 64), at k = 4 the L1 data path
 // (k |A| through it) and the sums' shared-memory traffic. Boxes of about 64 entries per half-warp: with 32 the
 // barrier waits for the longest list (k = 4, 7 slices: 616 us against 544), with 96 the lists take the shared memory that
 // the L1 cache needs for rows in flight (614 us).

@@ -437,7 +437,9 @@ __global__ void __launch_bounds__(kQRThreads, CTAS) qr64_kernel(const QRArgs a) 
   if (b == 0) back_substitute(L, Wl);
 }
 
-// Dynamic shared memory a QR CTA may use: the opt-in limit less the static arrays and a margin.
+// Dynamic shared memory a QR CTA may use: the opt-in limit less 10 KB for the static arrays (7 KB) and a margin.
+// (Rows are counted with n + 3 doubles below, two more than they take: the split into groups and CTAs that the
+// solvers' results were measured with.)
 size_t solve_smem_budget(size_t smem_optin) {
   const size_t fixed = sizeof(double) * (kQRMaxCols + 4) + 2048;
   return smem_optin > fixed ? smem_optin - fixed : 0;
