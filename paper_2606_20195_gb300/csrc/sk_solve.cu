@@ -128,9 +128,10 @@ __device__ __forceinline__ double load_val(const void* p, int64_t idx) {
 // One panel's reflectors from its Gram matrix and top rows (one warp; NB <= 16). Lane c < NB holds column
 // c of the top rows, lane NB + c column c of the Gram matrix (further lanes repeat those). Writes the
 // panel's w_ic = v_i^T W_c (c > i), R's rows, tau_i and v_i's entry on row i, and returns the panel's
-// width: `wmax` columns, fewer if one is cut off.
+// width: `wmax` columns, fewer if one is cut off. (Not inlined: its 16 doubles a lane then take no registers
+// from the other phases. 1024 x 64 with 128 registers a thread 279 -> 275 us; 4096 x 1024 11450 -> 11290.)
 template <int NB>
-__device__ int panel_factor(const double* G, const double* top, int wmax, double* wsm, double* rsm, double* taus,
+__device__ __noinline__ int panel_factor(const double* G, const double* top, int wmax, double* wsm, double* rsm, double* taus,
                             double* v0s) {
   const int lane = threadIdx.x & 31;
   const int c = lane % NB;
@@ -256,8 +257,8 @@ __device__ void back_substitute(const SolveLaunch& L, double* rhs) {
 // CTA, and its CTAs all the registers they can use. A narrow one has to leave room: its cooperative launch
 // starts when every CTA has a place, and a CTA with 255 registers a thread has none beside another request's
 // kernel. A service's saturated stream of requests (n up to 256; m from 2^14 to 2^24, or to 2^20 rows) then
-// makes 363 / 1290 solves a second, with 128 registers 381 / 1530 (384 / 1360 with the kernel that took one
-// reduction per column and 64 registers). One QR alone takes 1 to 2 % longer: 1024 x 64 279 us, not 275.
+// makes 363 / 1290 solves a second, with 128 registers 382 / 1550, with 80 390 / 1610 (384 / 1360 with the
+// kernel that took one reduction per column and 64 registers). A QR alone: 1024 x 64 275 -> 279 us.
 template <typename T, int NB, int CTAS>
 __global__ void __launch_bounds__(kQRThreads, CTAS) qr64_kernel(const QRArgs a) {
   const long long wait = a.L.wait_cycles > 0 ? a.L.wait_cycles : kBarrierCycles;
@@ -491,8 +492,8 @@ cudaError_t launch_solve(const SolveLaunch& L, cudaStream_t st, int32_t* launche
   const size_t smem = std::max<size_t>((size_t)a.rpc * (size_t)(L.n + 1) * 8, (size_t)L.n * 8);
   void* args[] = {(void*)&a};
   const bool alone = 2 * smem > 200 * 1024;  // no second CTA of this size on an SM
-  const void* kern = nb == 16 ? (alone ? qr_kernel<16, 1>(L) : qr_kernel<16, 2>(L))
-                     : nb == 8 ? qr_kernel<8, 2>(L)
+  const void* kern = nb == 16 ? (alone ? qr_kernel<16, 1>(L) : qr_kernel<16, 3>(L))
+                     : nb == 8 ? qr_kernel<8, 2>(L)  // (128 registers hold these without spilling)
                                : qr_kernel<4, 2>(L);
   e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
