@@ -579,7 +579,8 @@ sk_status validate_apply(const sk_plan_s* p, const void* A, int64_t lda, int64_t
 
 bool capturing(cudaStream_t st) {
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) return cudaGetLastError(), true;
+  return cap != cudaStreamCaptureStatusNone;
 }
 
 // Chunk-total bytes of a sketch with chunk length R.

@@ -138,8 +138,9 @@ def test_one_plan_on_several_streams(sk, dev, shape):
     plan.close()
 
 
-def test_eager_call_beside_another_streams_capture(sk, dev):
-    # The scratch of an eager call is allocated while another stream is being captured (global mode).
+@pytest.mark.parametrize("before", [64, 2000])  # rows of an earlier call: too few for totals, and some
+def test_eager_call_beside_another_streams_capture(sk, dev, before):
+    # The scratch of an eager call is allocated, or grown, while another stream is being captured (global mode).
     import torch
     m, n, d, k = 16384, 16, 256, 4
     A = _ints(m, n, 1)
@@ -148,8 +149,8 @@ def test_eager_call_beside_another_streams_capture(sk, dev):
     Y, Z = (torch.zeros((d, n), dtype=torch.float16, device=dev) for _ in range(2))
     side = torch.cuda.Stream()
     first.apply(Ad, Z)
-    small = torch.from_numpy(A[:64]).to(dev)
-    plan.set(sk.SK_PARAM_ROWS, 64)
+    small = torch.from_numpy(A[:before]).to(dev)
+    plan.set(sk.SK_PARAM_ROWS, before)
     plan.apply(small, Y)  # (the plan's status word)
     plan.set(sk.SK_PARAM_ROWS, m)
     torch.cuda.synchronize()
