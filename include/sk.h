@@ -132,11 +132,9 @@ typedef enum {
    * would grow the plan's scratch beyond it returns SK_ERR_OOM before enqueueing any work (Y is left
    * as it was); for services that admit work under a device-memory budget. */
   SK_PARAM_SCRATCH_LIMIT = 13,
-  /* Upper bound, in SM clock cycles, on each grid-barrier wait of sk_solve's QR kernel and of small
-   * sketches that finish in one launch (0, the default: about two seconds). A barrier that gives up ends
-   * the kernel and sk_solve_status returns SK_ERR_TIMEOUT (a sketch sets bit 0 of
-   * SK_PARAM_DEVICE_STATUS, its Y is invalid, and the next call is unaffected); small values exist to
-   * exercise that path. */
+  /* Upper bound, in SM clock cycles, on each grid-barrier wait of sk_solve's QR kernel (0, the
+   * default: about two seconds). A barrier that gives up ends the kernel and sk_solve_status returns
+   * SK_ERR_TIMEOUT; small values exist to exercise that path. */
   SK_PARAM_SOLVE_WAIT_CYCLES = 14,
   /* Read-only: bytes of device scratch the plan holds now. */
   SK_PARAM_SCRATCH_BYTES = 15,
@@ -150,7 +148,11 @@ typedef enum {
    * chunks per matrix and at least 4096 rows (a multiple of 256), instead of the tuning that looks at
    * the whole batch. A request's chunking, hence its rounding, then does not depend on what else is
    * in the batch (0, the default: tuned over the batch; SK_PARAM_CHUNK_ROWS, if set, wins). */
-  SK_PARAM_ITEM_CHUNKS = 17
+  SK_PARAM_ITEM_CHUNKS = 17,
+  /* The same bound for the grid barrier of small sketches that finish in one launch. A barrier that
+   * gives up sets bit 0 of SK_PARAM_DEVICE_STATUS and leaves that call's Y invalid; the plan's next
+   * call is unaffected. */
+  SK_PARAM_SKETCH_WAIT_CYCLES = 18
 } sk_param;
 
 enum { SK_MODE_ATOMIC = 0, SK_MODE_DETERMINISTIC = 1, SK_MODE_SERIAL_TILE = 2 };
@@ -197,7 +199,9 @@ SK_API sk_status sk_plan_get(sk_plan plan, int32_t key, int64_t* value);
  *   n      columns, 1 <= n <= 65535
  *   Y_dev  device, d x n, float (SK_FP32) or binary16 (FP16 rules), 4-byte aligned. Overwritten:
  *          the call zeroes Y on `stream` before accumulating.
- * The rows processed are the plan's m rows starting at global row SK_PARAM_ROW_OFFSET.
+ * The rows processed are the plan's m rows starting at global row SK_PARAM_ROW_OFFSET. Scratch (the
+ * status word, and chunk totals where the kernel taken uses them) is allocated on first use and grown as
+ * needed: above 1 MB that takes a call some 65 us once.
  */
 SK_API sk_status sk_apply(sk_plan plan, const float* A_dev, int64_t lda, int64_t n, void* Y_dev, void* stream);
 

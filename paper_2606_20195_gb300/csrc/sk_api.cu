@@ -56,7 +56,8 @@ struct sk_plan_s {
   int64_t solve_group_rows = 0;  // rows per QR group of sk_solve (0: as many as shared memory holds)
   int32_t list_cap = 0;          // register kernel: list entries per output row and box (0: automatic)
   int64_t scratch_limit = 0;     // bound on the plan's device scratch in bytes (0: none)
-  int64_t solve_wait_cycles = 0; // bound on each grid-barrier wait (0: default)
+  int64_t solve_wait_cycles = 0; // bound on each grid-barrier wait of the QR kernel (0: default)
+  int64_t sketch_wait_cycles = 0;  // and of one-launch sketches
   int64_t last_launches = 0, last_R = 0;
   int32_t last_kernel = 0;  // kernel of the last sketch: 1 tile, 2 literal, 3 owner, 4 global, 5 deterministic, 6 register, 7 gather
   bool last_noalloc = false;  // the last sketch was an sk_apply_noalloc call (status in the static array)
@@ -789,7 +790,7 @@ sk_status enqueue_sketch(sk_plan_s* p, const void* A, int64_t lda, int64_t n, in
   if (fast) {
     // The short slices finish in the same launch if Y is this call's alone (not one that other calls add to).
     if (zero_y && cfg.tile_alone()) L.bar = p->fastP;
-    L.wait_cycles = p->solve_wait_cycles;
+    L.wait_cycles = p->sketch_wait_cycles;
   } else if (cfg.slices > 1 || cfg.glob || cfg.reg || cfg.gat) {
     const size_t needP = sizeof(float) * (size_t)launch_P_floats(L);
     if (p->tileP_bytes < needP) {
@@ -903,6 +904,10 @@ sk_status sk_plan_set(sk_plan p, int32_t key, int64_t v) {
       if (v < 0) return set_error(SK_ERR_INVALID_ARG, "solve wait cycles must be >= 0");
       p->solve_wait_cycles = v;
       return SK_OK;
+    case SK_PARAM_SKETCH_WAIT_CYCLES:
+      if (v < 0) return set_error(SK_ERR_INVALID_ARG, "sketch wait cycles must be >= 0");
+      p->sketch_wait_cycles = v;
+      return SK_OK;
     default:
       return set_error(SK_ERR_INVALID_ARG, "unknown or read-only key %d", key);
   }
@@ -923,6 +928,7 @@ sk_status sk_plan_get(sk_plan p, int32_t key, int64_t* v) {
     case SK_PARAM_SCRATCH_LIMIT: *v = p->scratch_limit; return SK_OK;
     case SK_PARAM_ROWS: *v = p->m; return SK_OK;
     case SK_PARAM_SOLVE_WAIT_CYCLES: *v = p->solve_wait_cycles; return SK_OK;
+    case SK_PARAM_SKETCH_WAIT_CYCLES: *v = p->sketch_wait_cycles; return SK_OK;
     case SK_PARAM_SCRATCH_BYTES: *v = (int64_t)plan_scratch_bytes(p); return SK_OK;
     case SK_PARAM_LAST_LAUNCHES: *v = p->last_launches; return SK_OK;
     case SK_PARAM_LAST_CHUNK_ROWS: *v = p->last_R; return SK_OK;

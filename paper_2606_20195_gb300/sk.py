@@ -20,7 +20,7 @@ SK_PARAM_CHUNK_ROWS, SK_PARAM_MODE, SK_PARAM_ROW_OFFSET, SK_PARAM_KERNEL = 1, 2,
 SK_PARAM_TILE_COLS, SK_PARAM_THREADS, SK_PARAM_LAST_LAUNCHES, SK_PARAM_LAST_CHUNK_ROWS = 5, 6, 7, 8
 SK_PARAM_DEVICE_STATUS, SK_PARAM_LAST_KERNEL, SK_PARAM_SOLVE_GROUP_ROWS, SK_PARAM_LIST_CAP = 9, 10, 11, 12
 SK_PARAM_SCRATCH_LIMIT, SK_PARAM_SOLVE_WAIT_CYCLES, SK_PARAM_SCRATCH_BYTES, SK_PARAM_ROWS = 13, 14, 15, 16
-SK_PARAM_ITEM_CHUNKS = 17
+SK_PARAM_ITEM_CHUNKS, SK_PARAM_SKETCH_WAIT_CYCLES = 17, 18
 SK_MODE_ATOMIC, SK_MODE_DETERMINISTIC, SK_MODE_SERIAL_TILE = 0, 1, 2
 SK_KERNEL_AUTO, SK_KERNEL_TILE, SK_KERNEL_LITERAL, SK_KERNEL_OWNER, SK_KERNEL_GLOBAL = 0, 1, 2, 3, 4
 SK_KERNEL_REGISTER, SK_KERNEL_GATHER = 6, 7
@@ -274,7 +274,8 @@ class Plan:
         keys = {"chunk_rows": SK_PARAM_CHUNK_ROWS, "mode": SK_PARAM_MODE, "row_offset": SK_PARAM_ROW_OFFSET,
                 "kernel": SK_PARAM_KERNEL, "tile_cols": SK_PARAM_TILE_COLS, "threads": SK_PARAM_THREADS,
                 "solve_group_rows": SK_PARAM_SOLVE_GROUP_ROWS, "list_cap": SK_PARAM_LIST_CAP,
-                "scratch_limit": SK_PARAM_SCRATCH_LIMIT, "solve_wait_cycles": SK_PARAM_SOLVE_WAIT_CYCLES}
+                "scratch_limit": SK_PARAM_SCRATCH_LIMIT, "solve_wait_cycles": SK_PARAM_SOLVE_WAIT_CYCLES,
+                "sketch_wait_cycles": SK_PARAM_SKETCH_WAIT_CYCLES}
         for name, v in params.items():
             sk_plan_set(self.handle, keys[name], int(v))
 

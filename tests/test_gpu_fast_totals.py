@@ -69,12 +69,13 @@ def test_call_after_a_barrier_gave_up(sk, dev, shape):
     import torch
     m, n, d, k = shape
     A = _ints(m, n, 3)
-    plan = sk.Plan(d, m, k, 1, 11, solve_wait_cycles=1)
+    plan = sk.Plan(d, m, k, 1, 11, sketch_wait_cycles=1)
     Ad, Y = torch.from_numpy(A).to(dev), torch.empty((d, n), dtype=torch.float16, device=dev)
     for _ in range(3):
         plan.apply(Ad, Y)
     assert plan.get(sk.SK_PARAM_DEVICE_STATUS) == 1
-    plan.set(sk.SK_PARAM_SOLVE_WAIT_CYCLES, 0)
+    plan.set(sk.SK_PARAM_SKETCH_WAIT_CYCLES, 0)
+    plan.set(sk.SK_PARAM_SOLVE_WAIT_CYCLES, 1)  # (the QR's own bound)
     for _ in range(2):
         plan.apply(Ad, Y)
         torch.cuda.synchronize()
