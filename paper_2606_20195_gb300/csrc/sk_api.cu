@@ -611,7 +611,11 @@ template <typename T>
 bool grow_totals(sk_plan_s* p, T** ptr, size_t* cur, size_t need, cudaStream_t st) {
   if (*cur >= need) return true;
   if (plan_grow(p, ptr, cur, need, "chunk-total scratch") != SK_OK) return clear_error(), false;
-  return cudaMemsetAsync(*ptr, 0, need, st) == cudaSuccess;
+  if (cudaMemsetAsync(*ptr, 0, need, st) == cudaSuccess) return true;
+  cudaFree(*ptr);  // (not zero: must not be taken for totals by a later call)
+  *ptr = nullptr;
+  *cur = 0;
+  return cudaGetLastError(), false;
 }
 
 // The `need` bytes of chunk totals in p->fastP, for a sketch that can do without any; null where they are not to

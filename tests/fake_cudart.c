@@ -45,7 +45,11 @@ int cudaMalloc(void** p, size_t bytes) {
   return *p = malloc(64), OK;
 }
 int cudaFree(void* p) { return ++fake_frees, free(p), OK; }
-int cudaMemsetAsync(void* p, int v, size_t n, void* st) { return (void)p, (void)v, (void)n, (void)st, OK; }
+int fake_memset_fails = 0;
+int cudaMemsetAsync(void* p, int v, size_t n, void* st) {
+  (void)p, (void)v, (void)st;
+  return fake_memset_fails && n > 64 ? INVALID : OK;
+}
 int cudaMemcpyAsync(void* d, const void* s, size_t n, int kind, void* st) {
   (void)s, (void)st;
   if (kind == 2) memset(d, 0, n); /* device to host */

@@ -170,3 +170,16 @@ for (m, n, d, k), half in (((16384, 16, 256, 4), True), ((20000, 1, 256, 4), Tru
     assert apply(p, n) == (TILE, 1, 0)
     assert (grid.value <= 76) == half and grid.value >= 38, (m, n, grid.value)
 """)
+
+
+def test_totals_that_were_not_zeroed_are_not_kept(run):
+    run("""
+fails = var("fake_memset_fails")
+for case, n, t in ((GATH, 128, 0), (REG16, 64, 1)):
+    p = plan(case); fails.value = 1
+    try: apply(p, n, a_type=t)
+    except sk.SkError: pass  # (zeroing Y fails too)
+    fails.value = 0
+    assert held(p) == 4
+    assert apply(p, n, a_type=t)[0] in (GATHER, REG)
+""")
