@@ -72,10 +72,10 @@ __device__ __forceinline__ void df_add(float& s, float& c, float s2, float c2) {
 // c = (hi + lo) * scale with hi of magnitude 1/2 to 1 and scale a power of two (2^-120 to 2^120): lo keeps its
 // bits whatever c's exponent, where the second float of c itself would be subnormal from about 1e-31 down.
 __device__ __forceinline__ void split_scaled(double c, float& hi, float& lo, float& scale) {
-  int e = 0;
-  const double f = frexp(c, &e);
+  // (exponent and power of two by their bits: frexp and ldexp cost a pass 2 us of FP64 operations)
+  const int e = (int)(((unsigned)__double2hiint(c) >> 20) & 0x7FFu) - 1022;
   const int es = max(-120, min(120, e));
-  split_df(ldexp(f, e - es), hi, lo);
+  split_df(c * __hiloint2double((1023 - es) << 20, 0), hi, lo);
   scale = __uint_as_float((uint32_t)(es + 127) << 23);
 }
 
